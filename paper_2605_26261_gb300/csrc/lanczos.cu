@@ -12,9 +12,11 @@
 // queues 2 launches per step (3 for CR sectors, whose H.v launch leaves alpha_j
 // as per-tile sums for a short second launch), and a chain that breaks down
 // (beta_j <= tau) turns the rest of its launches into no-ops.
+#include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdlib>
-#include <atomic>
+#include <cstring>
 #include <mutex>
 #include <vector>
 
@@ -25,6 +27,7 @@
 #include "vec.cuh"
 #include "rng.cuh"
 #include "tridiag.cuh"
+#include "tridiag_dc.cuh"
 
 namespace ftlm {
 
@@ -179,14 +182,138 @@ __global__ void copy_meff_kernel(const ChainState *st, int B, int *dst)
     if (threadIdx.x < B) dst[threadIdx.x] = st[threadIdx.x].m_eff;
 }
 
+constexpr int kRitzThreads = 128;
+
 // Tridiagonal problems of this translation unit that did not converge (read and
 // cleared by ftlm_ritz_status); one copy per device.
 __device__ unsigned long long g_ritz_unconverged;
 
-// One thread per chain; T chains per CTA.  A chain whose QR iteration does not
-// converge within max_sweeps gets NaN Ritz values and weights.  rows == nullptr:
-// chain c reads row c of alpha/beta/mv and writes row c of theta/weight; else
-// rows[c] names its coefficient row and its outputs (and m_eff is copied out).
+// Coefficient row and outputs of chain c of a Ritz launch.  rows == nullptr: chain c
+// reads row c of alpha/beta/mv and writes row c of theta/weight; else rows[c] names
+// its coefficient row and its outputs (and m_eff is copied out).
+struct RitzIo {
+    size_t row;
+    double *theta, *weight;
+    int m;
+};
+__device__ __forceinline__ RitzIo ritz_io(int c, int M, const int *mv, double *theta, double *weight,
+                                          const RitzRow *rows, bool writer)
+{
+    RitzIo io;
+    if (rows) {
+        const RitzRow r = rows[c];
+        io.row = r.row;
+        io.theta = r.theta;
+        io.weight = r.weight;
+    } else {
+        io.row = (size_t)c;
+        io.theta = theta + io.row * M;
+        io.weight = weight + io.row * M;
+    }
+    const int m = mv[io.row];
+    if (rows && writer) rows[c].m_eff[0] = m;
+    io.m = m < 0 ? 0 : (m > M ? M : m);
+    return io;
+}
+
+// The Ritz step by divide and conquer (tridiag_dc.cuh), one CTA per chain; a chain's
+// results depend on its coefficients only, not on the launch.  A chain with a
+// non-finite coefficient or an unconverged root gets NaN Ritz values and weights.
+//
+// Bound: FP64 instructions on one SM per chain (two lanes per cycle).  One thread per
+// root of the merge; the whole problem lives in shared memory (88 bytes per row).
+__global__ void __launch_bounds__(kRitzThreads)
+ritz_dc_kernel(int M, const double *__restrict__ alpha, const double *__restrict__ beta, const int *__restrict__ mv,
+               double *theta, double *weight, const RitzRow *rows)
+{
+    extern __shared__ double sh[];
+    __shared__ unsigned long long s_max;  // largest |coefficient|, as bits (NaN above inf above all)
+    const int t = threadIdx.x, T = blockDim.x;
+    const RitzIo io = ritz_io(blockIdx.x, M, mv, theta, weight, rows, t == 0);
+    const int m = io.m;
+    const double *a = alpha + io.row * M, *b = beta + io.row * M;
+    bool ok = true;
+    dc::Work w = dc::carve(sh, m);
+    double back = 1.0;  // scale of the eigenvalues
+    if (m == 1) {
+        if (t == 0) {
+            w.d[0] = a[0];
+            w.f[0] = 1.0;
+        }
+        __syncthreads();
+    } else if (m > 1) {
+        if (t == 0) s_max = 0;
+        __syncthreads();
+        unsigned long long mx = 0;
+        for (int i = t; i < m; i += T) {
+            w.d[i] = a[i];
+            w.e[i] = i + 1 < m ? b[i] : 0.0;
+            mx = max(mx, (unsigned long long)__double_as_longlong(fabs(w.d[i])));
+            mx = max(mx, (unsigned long long)__double_as_longlong(fabs(w.e[i])));
+        }
+        atomicMax(&s_max, mx);
+        __syncthreads();
+        mx = s_max;
+        ok = mx < 0x7ff0000000000000ull;
+        if (ok) {  // uniform over the CTA
+            // an exact power of two brings the coefficients near one
+            const int ex = mx ? max(-1000, ilogb(__longlong_as_double((long long)mx))) : 0;
+            const double sc = ldexp(1.0, -ex);
+            back = ldexp(1.0, ex);
+            for (int i = t; i < m; i += T) {
+                w.d[i] *= sc;
+                w.e[i] *= sc;
+            }
+            dc::leaf_abs(w, t, T);
+            __syncthreads();
+            dc::leaf_tear(w, t, T);
+            __syncthreads();
+            for (int s = 1; s < m; s *= 2) {
+                dc::sort_block(w, s, t, T);
+                __syncthreads();
+                dc::mark_small(w, s, t, T);
+                __syncthreads();
+                dc::mark_pairs(w, s, t, T);
+                __syncthreads();
+                dc::deflate(w, s, t, T);
+                __syncthreads();
+                dc::float_images(w, t, T);
+                __syncthreads();
+                ok &= dc::roots(w, s, t, T);
+                __syncthreads();
+                dc::refit(w, s, t, T);
+                __syncthreads();
+                dc::rows(w, s, t, T);
+                __syncthreads();
+                dc::commit(w, t, T);
+                __syncthreads();
+            }
+        }
+        ok = __syncthreads_and(ok);
+        if (!ok && t == 0) atomicAdd(&g_ritz_unconverged, 1ull);
+    }
+    for (int k = t; k < M; k += T) {
+        if (k >= m || !ok) {
+            io.theta[k] = k < m ? NAN : 0.0;
+            io.weight[k] = k < m ? NAN : 0.0;
+        }
+    }
+    if (!ok) return;
+    for (int i = t; i < m; i += T) {  // ascending order
+        const long long key = dc::order_key(w.d[i]);
+        int r = 0;
+        for (int j = 0; j < m; ++j) {
+            const long long q = dc::order_key(w.d[j]);
+            r += (q < key) | ((q == key) & (j < i));
+        }
+        io.theta[r] = w.d[i] * back;
+        io.weight[r] = w.f[i] * w.f[i];
+    }
+}
+
+// The same by implicit QR with a sweep limit (ftlm_ritz_set_max_sweeps): one thread
+// per chain, T chains per CTA.  A chain whose iteration does not converge within
+// max_sweeps gets NaN Ritz values and weights.
 __global__ void ritz_kernel(int n, int M, const double *__restrict__ alpha, const double *__restrict__ beta,
                             const int *__restrict__ mv, double *theta, double *weight, const RitzRow *rows,
                             int max_sweeps)
@@ -196,21 +323,10 @@ __global__ void ritz_kernel(int n, int M, const double *__restrict__ alpha, cons
     const int c = blockIdx.x * T + i;
     if (c >= n) return;
     Strided d{sh + i, T}, e{sh + (size_t)M * T + i, T}, z{sh + (size_t)2 * M * T + i, T};
-    size_t row;
-    double *th, *wt;
-    if (rows) {
-        const RitzRow r = rows[c];
-        row = r.row;
-        th = r.theta;
-        wt = r.weight;
-    } else {
-        row = (size_t)c;
-        th = theta + row * M;
-        wt = weight + row * M;
-    }
-    int m = mv[row];
-    if (rows) rows[c].m_eff[0] = m;
-    m = m < 0 ? 0 : (m > M ? M : m);
+    const RitzIo io = ritz_io(c, M, mv, theta, weight, rows, true);
+    const size_t row = io.row;
+    double *th = io.theta, *wt = io.weight;
+    const int m = io.m;
     for (int k = 0; k < m; ++k) {
         d[k] = alpha[row * M + k];
         e[k] = k + 1 < m ? beta[row * M + k] : 0.0;
@@ -239,15 +355,26 @@ ftlm_status ritz_launch(int n, int M, const double *alpha, const double *beta, c
                         double *weight, const RitzRow *rows, cudaStream_t stream)
 {
     if (n == 0) return FTLM_OK;
-    constexpr size_t kSmemMax = 96 * 1024;
     int occ = 1;
+    const int max_sweeps = ritz_max_sweeps();
+    if (max_sweeps <= 0) {
+        // one thread per row up to kRitzThreads; the choice changes no result
+        const int T = std::min(kRitzThreads, (M + 31) / 32 * 32);
+        FTLM_CUDA(kernel_occupancy((const void *)ritz_dc_kernel, kRitzThreads, dc::kBytesPerRow * FTLM_MAX_LANCZOS,
+                                   true, &occ));
+        ritz_dc_kernel<<<n, T, dc::kBytesPerRow * M, stream>>>(M, alpha, beta, mv, theta, weight, rows);
+        note_launch();
+        FTLM_CUDA(cudaGetLastError());
+        return FTLM_OK;
+    }
+    constexpr size_t kSmemMax = 96 * 1024;
     FTLM_CUDA(kernel_occupancy((const void *)ritz_kernel, 32, kSmemMax, true, &occ));
     const size_t per_chain = 3 * (size_t)M * sizeof(double);
     int T = (int)(kSmemMax / per_chain);
     T = T < 1 ? 1 : (T > 32 ? 32 : T);
     if (T > n) T = n;
     const int grid = (n + T - 1) / T;
-    ritz_kernel<<<grid, T, per_chain * T, stream>>>(n, M, alpha, beta, mv, theta, weight, rows, ritz_max_sweeps());
+    ritz_kernel<<<grid, T, per_chain * T, stream>>>(n, M, alpha, beta, mv, theta, weight, rows, max_sweeps);
     note_launch();
     FTLM_CUDA(cudaGetLastError());
     return FTLM_OK;
