@@ -13,10 +13,15 @@
 //    a fixed order and stores alpha_j (epi_end);
 //  - dynamic tile order (CR launches: tiles handed out by a counter, so that all
 //    warps work on one frontier of rows and the gathers of the rows in flight
-//    share L2): each tile's sums go through a fixed warp tree into a slot of their
-//    own (store_tile), and a second launch adds the slots in tile order.
-// Both orders are fixed for a given sector and grid: alpha_j is reproducible.
+//    share L2): each tile's sums go through a fixed warp tree and are added as whole
+//    numbers of two words (AlphaSums), whose sum does not depend on the order; a
+//    launch of one warp turns it into alpha_j.  A slot per tile, added in tile order by
+//    a second launch, cost 15 to 41 us per step and 2 B bytes per row.
+// Either way the result is fixed for a given sector and grid: alpha_j is reproducible.
 #pragma once
+
+#include <algorithm>
+#include <cmath>
 
 #include "ftlm_internal.cuh"
 #include "reduce.cuh"
@@ -27,9 +32,11 @@ namespace ftlm {
 struct EpiDev {
     ChainState *st;
     double *partials;
-    unsigned int *counter;  // [0] block ticket; [1], [2] dynamic tile order
+    unsigned int *counter;  // [0] block ticket; [1], [2], [3] dynamic tile order
     double *alpha_out;
-    double *tile_part;      // per-tile sums of the dynamic tile order, [tile][B]
+    unsigned long long *fixed;  // sums of the dynamic tile order, two words per chain
+    double scale[2], unscale[2];  // 2^alpha_shift and 2^-alpha_shift as products of two factors:
+                                  // the first word of a sum counts 2^-alpha_shift
     int alpha_stride;
     int has_prev;
 };
@@ -42,7 +49,14 @@ inline EpiDev epi_of(const LanczosHv *epi)
         ep.partials = epi->partials;
         ep.counter = epi->counter;
         ep.alpha_out = epi->alpha_out;
-        ep.tile_part = epi->tile_part;
+        ep.fixed = epi->fixed;
+        // |alpha_j| <= ||H|| < 2^e: counting 2^-(60 - e) keeps the sum below 2^60
+        const int e = epi->norm_bound > 0.0 ? std::ilogb(epi->norm_bound) + 1 : 0;
+        const int shift = 60 - e;
+        ep.scale[0] = std::ldexp(1.0, shift / 2);
+        ep.scale[1] = std::ldexp(1.0, shift - shift / 2);
+        ep.unscale[0] = 1.0 / ep.scale[0];
+        ep.unscale[1] = 1.0 / ep.scale[1];
         ep.alpha_stride = epi->alpha_stride;
         ep.has_prev = epi->j > 1;
     }
@@ -116,42 +130,21 @@ __device__ __forceinline__ void epi_row_walk_a(const EpiDev &ep, const V *s_inv_
 template <typename V, int B, int THREADS>
 __device__ __forceinline__ void epi_end(const EpiDev &ep, DotAcc<V> (&apart)[B])
 {
-    __shared__ double s_part[B];
-#pragma unroll
-    for (int r = 0; r < B; ++r) {
-        const double part = block_sum<THREADS>(apart[r].value());
-        if (threadIdx.x == 0) s_part[r] = part;
-    }
-    __syncthreads();
-    bool last = false;
-    {
-        __shared__ bool s_last;
-        if (threadIdx.x == 0) {
-#pragma unroll
-            for (int r = 0; r < B; ++r) ep.partials[(size_t)blockIdx.x * B + r] = s_part[r];
-            __threadfence();
-            s_last = atomicAdd(ep.counter, 1u) == gridDim.x - 1;
-        }
-        __syncthreads();
-        last = s_last;
-    }
-    if (last && threadIdx.x < 32) {
-        for (int r = 0; r < B; ++r) {
-            double v = 0.0;
-            for (int g = threadIdx.x; g < (int)gridDim.x; g += 32) v += __ldcg(ep.partials + (size_t)g * B + r);
-            v = warp_sum(v);
-            if (threadIdx.x == 0 && !ep.st[r].stopped) {
-                ep.st[r].alpha = v;
-                ep.alpha_out[(size_t)r * ep.alpha_stride] = v;
-            }
-        }
+    const double part = block_sums<V, B, THREADS>(apart);
+    if (publish_sums<B>(part, ep.partials, ep.counter)) {
+        totals<B, THREADS>(ep.partials, gridDim.x, [&](int r, double v) {
+            if (ep.st[r].stopped) return;
+            ep.st[r].alpha = v;
+            ep.alpha_out[(size_t)r * ep.alpha_stride] = v;
+        });
         if (threadIdx.x == 0) *ep.counter = 0;
     }
 }
 
 // Dynamic tile order: a warp's first tile is its index, later ones come from the
-// counter ep.counter[1]; ep.counter[2] counts the warps that ran out of tiles, and
-// the last of them zeroes both for the next launch (they start at zero).  A warp
+// counter ep.counter[1], which is zero when a launch starts: alpha_kernel zeroes it at
+// the end of a step, and walk A's last warp to run out of tiles (ep.counter[2] counts
+// them) for the walk B that follows.  A warp
 // claims its next tile when it starts a tile (claim_tile, lane 0) and reads the
 // claim when it finishes (claimed_tile), so the atomic's round trip is hidden.
 __device__ __forceinline__ uint32_t claim_tile(const EpiDev &ep)
@@ -164,6 +157,58 @@ __device__ __forceinline__ uint32_t claimed_tile(uint32_t claim, uint32_t nwarps
     return __shfl_sync(0xffffffffu, claim, 0) + nwarps;
 }
 
+// Sums of per-tile values as whole numbers of two words, one pair per warp and chain in
+// shared memory: the first word counts 2^-alpha_shift, the second 2^-(alpha_shift +
+// 40).  Every value is taken to 2^-(alpha_shift + 40), about 2^-100 ||H||, and whole
+// numbers add in any order to the same sum, so the warps may take their tiles in any
+// order.  bad: bit r is set when a value of chain r was not finite.
+template <int B, int THREADS> struct AlphaSums {
+    long long v[THREADS / 32][2 * B];
+    unsigned int bad;
+};
+
+// Before the launch's first barrier, by every thread.
+template <int B, int THREADS> __device__ __forceinline__ void tiles_begin(AlphaSums<B, THREADS> &s)
+{
+    for (int i = threadIdx.x; i < THREADS / 32 * 2 * B; i += THREADS) s.v[i / (2 * B)][i % (2 * B)] = 0;
+    if (threadIdx.x == 0) s.bad = 0;
+}
+
+// Adds the warp's alpha partial sums of one tile, through a fixed warp tree.  Called by
+// the whole warp.
+template <typename V, int B, int THREADS>
+__device__ __forceinline__ void add_tile(const EpiDev &ep, AlphaSums<B, THREADS> &s, DotAcc<V> (&a)[B])
+{
+    const DotAcc<V> t = warp_sum_multi<V, B>(a);
+    const unsigned lane = threadIdx.x & 31u;
+    if (lane < B) {
+        const int r = warp_multi_index<B>(lane);
+        long long *w = s.v[threadIdx.x >> 5] + 2 * r;
+        const double v = t.value() * ep.scale[0] * ep.scale[1];
+        const double h = rint(v);
+        if (!(fabs(v) < 0x1p62)) atomicOr(&s.bad, 1u << r);
+        w[0] += (long long)h;
+        w[1] += (long long)rint((v - h) * 0x1p40);
+    }
+}
+
+// End of a launch with the dynamic tile order, called by every thread: the CTA's
+// sums, one atomic addition per chain and word.  alpha_kernel (hv.cu) turns them into
+// alpha_j and zeroes the sums and the tile counter for the next step.
+template <int B, int THREADS>
+__device__ __forceinline__ void tiles_done(const EpiDev &ep, AlphaSums<B, THREADS> &s)
+{
+    __syncthreads();
+    if (threadIdx.x < 2 * B) {
+        long long v = 0;
+#pragma unroll
+        for (int w = 0; w < THREADS / 32; ++w) v += s.v[w][threadIdx.x];
+        atomicAdd(&ep.fixed[threadIdx.x], (unsigned long long)v);
+        if (threadIdx.x == 0 && s.bad) atomicOr(ep.counter + 3, s.bad);
+    }
+}
+
+// End of a launch that takes its tiles in dynamic order and leaves no sums (walk A).
 __device__ __forceinline__ void tiles_done(const EpiDev &ep, uint32_t nwarps)
 {
     if ((threadIdx.x & 31u) == 0) {
@@ -173,16 +218,6 @@ __device__ __forceinline__ void tiles_done(const EpiDev &ep, uint32_t nwarps)
             ep.counter[2] = 0;
         }
     }
-}
-
-// The warp's alpha partial sums of one tile, through a fixed warp tree, into
-// ep.tile_part[tile * B + r].  Called by the whole warp.
-template <typename V, int B>
-__device__ __forceinline__ void store_tile(const EpiDev &ep, uint32_t tile, DotAcc<V> (&a)[B])
-{
-    const DotAcc<V> t = warp_sum_multi<V, B>(a);
-    const unsigned lane = threadIdx.x & 31u;
-    if (lane < B) ep.tile_part[(size_t)tile * B + warp_multi_index<B>(lane)] = t.value();
 }
 
 }  // namespace ftlm

@@ -254,8 +254,11 @@ struct LanczosHv {
     double *alpha_out;     // alpha_j of chain r goes to alpha_out[r * alpha_stride]
     int alpha_stride;
     int j;
-    double *tile_part;     // [hv_lanczos_tiles() * B]: per-tile sums of a dynamic tile order
+    unsigned long long *fixed;  // kAlphaFixedBytes, zero between launches: alpha sums of a dynamic tile order
+    double norm_bound;     // upper bound of ||H||
 };
+// Two words per chain of a block (epi.cuh).
+constexpr uint64_t kAlphaFixedBytes = 2 * kMaxBlock * sizeof(unsigned long long);
 // General-spin counterparts (spin.cu) of the H.v launch and the label/rank kernels.
 ftlm_status launch_hv_spin(const ftlm_basis *b, ftlm_dtype dtype, int B, const void *x, void *y,
                            const LanczosHv *epi, cudaStream_t stream);
@@ -274,8 +277,8 @@ bool valid_block(int B);
 // FTLM_RANK_AUTO picks CR for sectors of at least this many rows.
 constexpr uint64_t kAutoCrRows = 1ull << 20;
 // Upper bound on the tiles of a Lanczos H.v launch of B vectors that takes its tiles
-// in dynamic order and leaves alpha_j as per-tile sums in LanczosHv::tile_part (CR
-// rank mode, one walk or split); 0 when the launch finishes alpha_j itself.
+// in dynamic order (CR rank mode, one walk or split), at least one; 0 for the others.
+// The workspace has B doubles per tile for it.
 uint32_t hv_lanczos_tiles(const ftlm_basis *b, int B);
 
 // ---- split Lanczos H.v (basis.cu, walkb.cu, hv.cu) -------------------------
@@ -284,7 +287,7 @@ uint32_t hv_lanczos_tiles(const ftlm_basis *b, int B);
 // more than kMaxHiBonds of them).
 bool build_hi_walk(const ftlm_basis *b, int rh, HiWalk *w);
 struct EpiDev;
-// Walk B of a split Lanczos step (the epilogue's alpha as per-tile sums).
+// Walk B of a split Lanczos step (finishes the rows and alpha).
 ftlm_status launch_walk_b(const ftlm_basis *b, const HiWalk &w, ftlm_dtype dtype, int B, const void *x, void *y,
                           const EpiDev &ep, cudaStream_t stream);
 // Walk A's tile layout (false when the sector has no walk A tile table).

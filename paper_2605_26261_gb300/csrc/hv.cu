@@ -20,7 +20,8 @@
 // launches hand them out from a counter, which keeps the warps on one frontier
 // of rows (they drift apart under the round-robin order, and the union of the
 // gather windows outgrows L2: 20 % fewer DRAM bytes, 25 % less time on the N = 30
-// icosahedral sector).  Their alpha sums are then finished per tile (epi.cuh).
+// icosahedral sector).  Their alpha sums are then added per tile as whole
+// numbers (epi.cuh).
 //
 // Two rank strategies:
 //   CLT  label n_t = basis[t]; rank(n') = C_b + popc(M_b & (2^j - 1)) with
@@ -84,12 +85,14 @@ hv_kernel(const SectorTables s, const BondList bl, const V *__restrict__ x, V *y
 {
     constexpr bool LANCZOS = EPI != kPlain;
     // CR Lanczos launches take their tiles in dynamic order (their gathers gain the
-    // most from a narrow frontier of rows) and store per-tile alpha sums
+    // most from a narrow frontier of rows) and add their alpha sums per tile
     constexpr bool TILES = LANCZOS && !CLT;
     extern __shared__ uint16_t s_tlo[];
     __shared__ uint4 s_bond[kMaxBondSlots];
     __shared__ V s_inv_s[B], s_c_prev[B];  // per-chain scalars of the epilogue
+    __shared__ AlphaSums<TILES ? B : 1, kRowThreads> s_asum;
     if (LANCZOS && epi_begin<V, B>(ep, s_inv_s, s_c_prev)) return;
+    if constexpr (TILES) tiles_begin(s_asum);
     {
         const uint4 *src = sizeof(V) == 4 ? bl.slots_f32 : bl.slots_f64;
         for (int i = threadIdx.x; i < bl.nb; i += blockDim.x) s_bond[i] = src[i];
@@ -128,7 +131,7 @@ hv_kernel(const SectorTables s, const BondList bl, const V *__restrict__ x, V *y
 #pragma unroll
             for (int i = 0; i < RT; ++i)
                 if (ok[i]) epi_row<V, B, true>(ep, s_inv_s, s_c_prev, x, y, t[i], jsum4 - dsum[i], acc[i], tacc);
-            store_tile<V, B>(ep, tile, tacc);
+            add_tile<V, B>(ep, s_asum, tacc);
         } else {
 #pragma unroll
             for (int i = 0; i < RT; ++i)
@@ -141,28 +144,30 @@ hv_kernel(const SectorTables s, const BondList bl, const V *__restrict__ x, V *y
         do_tile(tile);
         tile = TILES ? claimed_tile(claim, nwarps) : tile + nwarps;
     }
-    if (TILES) tiles_done(ep, nwarps);
-    else if (LANCZOS) epi_end<V, B, kRowThreads>(ep, apart);
+    if constexpr (TILES) tiles_done(ep, s_asum);
+    else if constexpr (LANCZOS) epi_end<V, B, kRowThreads>(ep, apart);
 }
 
-// alpha_j of a dynamically ordered launch from its per-tile sums: block b adds a
-// fixed range of tiles (each thread its tiles in order), then the block trees and
-// the last block's sum over the blocks in order (epi_end).  The grid depends only
-// on the tile count, so alpha_j is reproducible.
-template <int B>
-__global__ void __launch_bounds__(kRowThreads) tile_alpha_kernel(const EpiDev ep, uint32_t ntiles)
+// alpha_j of a dynamically ordered launch from its sums (epi.cuh); one warp.
+template <int B> __global__ void __launch_bounds__(32) alpha_kernel(const EpiDev ep)
 {
-    bool all_stopped = true;
-#pragma unroll
-    for (int r = 0; r < B; ++r) all_stopped &= ep.st[r].stopped != 0;
-    if (all_stopped) return;  // as the H.v launch: uniform over the grid
-    const uint32_t per = (ntiles + gridDim.x - 1) / gridDim.x;
-    const uint32_t t0 = min(ntiles, blockIdx.x * per), t1 = min(ntiles, t0 + per);
-    DotAcc<double> a[B];
-    for (uint32_t t = t0 + threadIdx.x; t < t1; t += blockDim.x)
-#pragma unroll
-        for (int r = 0; r < B; ++r) a[r].v += __ldcg(ep.tile_part + (size_t)t * B + r);
-    epi_end<double, B, kRowThreads>(ep, a);
+    const int r = threadIdx.x;
+    if (r < B) {
+        const long long hi = (long long)ep.fixed[2 * r], lo = (long long)ep.fixed[2 * r + 1];
+        const bool bad = (ep.counter[3] >> r) & 1u;
+        const double v = ((double)hi + (double)lo * 0x1p-40) * ep.unscale[0] * ep.unscale[1];
+        ep.fixed[2 * r] = 0;
+        ep.fixed[2 * r + 1] = 0;
+        if (!ep.st[r].stopped) {
+            ep.st[r].alpha = bad ? NAN : v;
+            ep.alpha_out[(size_t)r * ep.alpha_stride] = bad ? NAN : v;
+        }
+    }
+    __syncwarp();
+    if (r == 0) {
+        ep.counter[1] = 0;
+        ep.counter[3] = 0;
+    }
 }
 
 // Rows per thread (RT) for single vectors.  Measured on GB300 (icosidodecahedron,
@@ -240,15 +245,6 @@ ftlm_status launch_rows(const ftlm_basis *b, const BondList &bl, const V *x, V *
     return FTLM_OK;
 }
 
-// alpha_j from the per-tile sums of a dynamically ordered launch.
-template <int B>
-void launch_tile_alpha(const ftlm_basis *b, const EpiDev &ep, uint32_t ntiles, cudaStream_t stream)
-{
-    const int ga = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)b->num_sms * 2, (ntiles + 2047) / 2048));
-    tile_alpha_kernel<B><<<ga, kRowThreads, 0, stream>>>(ep, ntiles);
-    note_launch();
-}
-
 template <typename V, typename Lbl, bool CLT, bool LANCZOS, int RT, int B, int C>
 ftlm_status launch(const ftlm_basis *b, const V *x, V *y, const EpiDev &ep, cudaStream_t stream)
 {
@@ -256,22 +252,21 @@ ftlm_status launch(const ftlm_basis *b, const V *x, V *y, const EpiDev &ep, cuda
     ftlm_status st = FTLM_OK;
     if constexpr (LANCZOS && !CLT) {
         // CR Lanczos step: one walk over the rows, or the split (walk A, then walk B
-        // over the high-high bonds in the transposed order); alpha_j from per-tile sums
+        // over the high-high bonds in the transposed order)
         HiWalk w;
-        uint32_t ntiles;
         if (split_walks(b, B, sizeof(V), &w)) {
             const ftlm_dtype dt = sizeof(V) == 4 ? FTLM_F32 : FTLM_F64;
             LoWalk la;
             st = build_lo_walk(b, &la) ? launch_walk_a(b, la, dt, B, x, y, ep, stream)
                                        : fail(FTLM_EUNSUPPORTED, "split H.v without a walk A tile table");
             if (st == FTLM_OK) st = launch_walk_b(b, w, dt, B, x, y, ep, stream);
-            ntiles = w.ntiles;
         } else {
             st = launch_rows<V, Lbl, false, kLanczos, RT, B, C>(b, b->bonds_cr, x, y, ep, stream);
-            const uint64_t rows = 32ull * RT;
-            ntiles = (uint32_t)((b->D + rows - 1) / rows);
         }
-        if (st == FTLM_OK) launch_tile_alpha<B>(b, ep, ntiles, stream);
+        if (st == FTLM_OK) {
+            alpha_kernel<B><<<1, 32, 0, stream>>>(ep);
+            note_launch();
+        }
     } else {
         st = launch_rows<V, Lbl, CLT, LANCZOS ? kLanczos : kPlain, RT, B, C>(b, CLT ? b->bonds_clt : b->bonds_cr, x,
                                                                            y, ep, stream);

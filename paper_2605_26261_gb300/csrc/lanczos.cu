@@ -9,9 +9,9 @@
 // and publishes beta_j.  The division by beta_j is folded into the next H.v (the
 // stored vectors stay un-normalized, q_j = u_j / s_j), so every step streams each
 // vector exactly once per launch.  All scalars stay on the device; the host only
-// queues 2 launches per step (3 for CR sectors, whose H.v launch leaves alpha_j
-// as per-tile sums for a short second launch), and a chain that breaks down
-// (beta_j <= tau) turns the rest of its launches into no-ops.
+// queues 2 launches per step (3 for CR sectors, whose H.v launch leaves the sums of
+// alpha_j for a launch of one warp, 4 where it runs as two walks), and a chain that
+// breaks down (beta_j <= tau) turns the rest of its launches into no-ops.
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -37,38 +37,6 @@ struct Keys {
     uint64_t k[kMaxBlock];
 };
 
-// Finish a launch's per-chain reduction: every block stores its B partial sums;
-// the last block to arrive returns true (in every thread) and the caller's warp 0
-// adds the partials of chain r in block order with chain_total().
-template <int B>
-__device__ __forceinline__ bool publish_partials(const double (&part)[B], double *partials, unsigned int *counter)
-{
-    __shared__ double s_part[B];
-    __shared__ bool s_last;
-#pragma unroll
-    for (int r = 0; r < B; ++r) {
-        const double v = block_sum<kRowThreads>(part[r]);
-        if (threadIdx.x == 0) s_part[r] = v;
-    }
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int r = 0; r < B; ++r) partials[(size_t)blockIdx.x * B + r] = s_part[r];
-        __threadfence();
-        s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    return s_last;
-}
-
-// Fixed-order total of chain r's partials; call from warp 0, valid in lane 0.
-template <int B>
-__device__ __forceinline__ double chain_total(const double *partials, int r)
-{
-    double v = 0.0;
-    for (int g = threadIdx.x; g < (int)gridDim.x; g += 32) v += __ldcg(partials + (size_t)g * B + r);
-    return warp_sum(v);
-}
-
 // Start vectors of a block of B chains (generated, or copied from src rows of
 // length D), interleaved, and s_1 = ||u|| of each chain's stored (dtype-rounded)
 // entries.
@@ -89,22 +57,18 @@ start_kernel(uint32_t D, const Keys keys, int dist, const double *__restrict__ s
         }
         st_vec<B>(u + (size_t)t * B, out);
     }
-    double part[B];
-#pragma unroll
-    for (int r = 0; r < B; ++r) part[r] = acc[r].value();
-    if (publish_partials<B>(part, partials, counter) && threadIdx.x < 32) {
-        for (int r = 0; r < B; ++r) {
-            const double nrm = sqrt(chain_total<B>(partials, r));
-            if (threadIdx.x == 0) {
-                ChainState &c = st[r];
-                c.s_cur = nrm;
-                c.s_prev = 1.0;
-                c.beta_prev = 0.0;
-                c.alpha = 0.0;
-                c.m_eff = 0;
-                c.stopped = (nrm > 0.0 && isfinite(nrm)) ? 0 : 1;
-            }
-        }
+    const double v = block_sums<V, B, kRowThreads>(acc);
+    if (publish_sums<B>(v, partials, counter)) {
+        totals<B, kRowThreads>(partials, gridDim.x, [&](int r, double sum) {
+            const double nrm = sqrt(sum);
+            ChainState &c = st[r];
+            c.s_cur = nrm;
+            c.s_prev = 1.0;
+            c.beta_prev = 0.0;
+            c.alpha = 0.0;
+            c.m_eff = 0;
+            c.stopped = (nrm > 0.0 && isfinite(nrm)) ? 0 : 1;
+        });
         if (threadIdx.x == 0) *counter = 0;
     }
 }
@@ -117,14 +81,25 @@ __global__ void __launch_bounds__(kRowThreads)
 update_kernel(uint32_t D, V *__restrict__ y, const V *__restrict__ u, ChainState *st, double *partials,
               unsigned int *counter, int j, int m_max, double tau, double *beta_out, int beta_stride)
 {
+    // the per-chain scalars once per CTA: a division in every thread is 10 FP64
+    // instructions per chain on a pipe of two lanes per cycle (40 us per launch at B = 8,
+    // whatever D)
+    __shared__ V s_a[B];
+    __shared__ int s_zero[B];
+    if (threadIdx.x < B) {
+        const ChainState &c = st[threadIdx.x];
+        s_zero[threadIdx.x] = c.stopped;
+        s_a[threadIdx.x] = c.stopped ? (V)0 : (V)(c.alpha / c.s_cur);
+    }
+    __syncthreads();
     V a[B];
     bool zero[B];
     bool all_stopped = true;
 #pragma unroll
     for (int r = 0; r < B; ++r) {
-        zero[r] = st[r].stopped != 0;
+        zero[r] = s_zero[r] != 0;
         all_stopped &= zero[r];
-        a[r] = zero[r] ? (V)0 : (V)(st[r].alpha / st[r].s_cur);
+        a[r] = s_a[r];
     }
     if (all_stopped) return;
     constexpr int W = 16 / (int)sizeof(V);
@@ -150,29 +125,26 @@ update_kernel(uint32_t D, V *__restrict__ y, const V *__restrict__ u, ChainState
         y[e] = w;
         acc[0].add(w, w);
     }
-    double part[B];
-#pragma unroll
-    for (int r = 0; r < B; ++r) part[r] = acc[r].value();
-    if (publish_partials<B>(part, partials, counter) && threadIdx.x < 32) {
-        for (int r = 0; r < B; ++r) {
-            const double beta = sqrt(chain_total<B>(partials, r));
-            if (threadIdx.x == 0 && !st[r].stopped) {
-                ChainState &c = st[r];
-                if (j < m_max) {
-                    if (beta <= tau) {
-                        c.stopped = 1;
-                        c.m_eff = j;
-                    } else {
-                        beta_out[(size_t)r * beta_stride + (j - 1)] = beta;
-                        c.s_prev = c.s_cur;
-                        c.s_cur = beta;
-                        c.beta_prev = beta;
-                    }
+    const double v = block_sums<V, B, kRowThreads>(acc);
+    if (publish_sums<B>(v, partials, counter)) {
+        totals<B, kRowThreads>(partials, gridDim.x, [&](int r, double sum) {
+            ChainState &c = st[r];
+            if (c.stopped) return;
+            const double bt = sqrt(sum);
+            if (j < m_max) {
+                if (bt <= tau) {
+                    c.stopped = 1;
+                    c.m_eff = j;
                 } else {
-                    c.m_eff = m_max;
+                    beta_out[(size_t)r * beta_stride + (j - 1)] = bt;
+                    c.s_prev = c.s_cur;
+                    c.s_cur = bt;
+                    c.beta_prev = bt;
                 }
+            } else {
+                c.m_eff = m_max;
             }
-        }
+        });
         if (threadIdx.x == 0) *counter = 0;
     }
 }
@@ -452,7 +424,7 @@ Layout layout(const ftlm_basis *b, int R, int M, ftlm_dtype dtype, int bmax = 0)
     l.beta = l.alpha + align256((uint64_t)R * M * sizeof(double));
     l.meff = l.beta + align256((uint64_t)R * M * sizeof(double));
     l.tiles = l.meff + align256((uint64_t)R * sizeof(int));
-    // per-tile alpha sums of dynamically ordered H.v launches (B >= 4 has the most tiles)
+    // alpha sums of dynamically ordered H.v launches (kAlphaFixedBytes of it are used)
     l.total = l.tiles + align256((uint64_t)hv_lanczos_tiles(b, 4) * l.bw * sizeof(double));
     return l;
 }
@@ -481,6 +453,7 @@ ftlm_status run_block(const ftlm_basis *b, int M, int r0, int chain0, uint64_t s
     const int g_upd = row_grid(b, ((uint64_t)D * B + U - 1) / U, occ_upd);
 
     FTLM_CUDA(cudaMemsetAsync(st, 0, lay.bw * sizeof(ChainState) + 64, stream));
+    if (lay.total > lay.tiles) FTLM_CUDA(cudaMemsetAsync(ws + lay.tiles, 0, kAlphaFixedBytes, stream));
     Keys keys{};
     for (int r = 0; r < B; ++r) keys.k[r] = chain_key(seed, b->key_n, b->K, (uint32_t)(chain0 + r0 + r));
     start_kernel<V, B><<<g_start, kRowThreads, 0, stream>>>(D, keys, dist, src ? src + (size_t)r0 * D : nullptr,
@@ -489,7 +462,8 @@ ftlm_status run_block(const ftlm_basis *b, int M, int r0, int chain0, uint64_t s
     FTLM_CUDA(cudaGetLastError());
     int cur = 0;
     for (int j = 1; j <= m_max; ++j) {
-        LanczosHv epi{st, partials, counter, alpha_ws + (size_t)r0 * M + (j - 1), M, j, (double *)(ws + lay.tiles)};
+        LanczosHv epi{st, partials, counter, alpha_ws + (size_t)r0 * M + (j - 1), M, j,
+                      (unsigned long long *)(ws + lay.tiles), b->tau64 * (0x1p53 / 100.0)};
         ftlm_status s = launch_hv(b, dtype, B, vec[cur], vec[1 - cur], &epi, stream);
         if (s != FTLM_OK) return s;
         void *tok = profile_begin(kProfUpdate, stream);

@@ -70,15 +70,6 @@ __device__ __forceinline__ bool tile_publish(DotAcc<V> (&acc)[B], double *partia
     return s_last;
 }
 
-// Fixed-order total of chain r over the unit's tiles; warp 0, valid in lane 0.
-template <int B>
-__device__ __forceinline__ double tile_total(const double *partials, uint32_t n_tiles, int r)
-{
-    double v = 0.0;
-    for (uint32_t k = threadIdx.x; k < n_tiles; k += 32) v += __ldcg(partials + (size_t)k * B + r);
-    return warp_sum(v);
-}
-
 // Start vectors of the units with j0 == jstart (every unit of a batch: jstart = 0).
 template <typename V, int B>
 __global__ void __launch_bounds__(kRowThreads)
@@ -105,20 +96,17 @@ ms_start_kernel(const MsUnit *__restrict__ units, const uint32_t *__restrict__ t
             }
             st_vec<B>(u0 + (size_t)t * B, out);
         }
-        if (tile_publish<V, B>(acc, uv.partials(), k, uv.counter(), U.n_stiles) && threadIdx.x < 32) {
-            ChainState *st = uv.st();
-            for (int r = 0; r < B; ++r) {
-                const double nrm = sqrt(tile_total<B>(uv.partials(), U.n_stiles, r));
-                if (threadIdx.x == 0) {
-                    ChainState &c = st[r];
-                    c.s_cur = nrm;
-                    c.s_prev = 1.0;
-                    c.beta_prev = 0.0;
-                    c.alpha = 0.0;
-                    c.m_eff = 0;
-                    c.stopped = (r < U.nact && nrm > 0.0 && isfinite(nrm)) ? 0 : 1;
-                }
-            }
+        if (tile_publish<V, B>(acc, uv.partials(), k, uv.counter(), U.n_stiles)) {
+            totals<B, kRowThreads>(uv.partials(), U.n_stiles, [&](int r, double sum) {
+                const double nrm = sqrt(sum);
+                ChainState &c = uv.st()[r];
+                c.s_cur = nrm;
+                c.s_prev = 1.0;
+                c.beta_prev = 0.0;
+                c.alpha = 0.0;
+                c.m_eff = 0;
+                c.stopped = (r < U.nact && nrm > 0.0 && isfinite(nrm)) ? 0 : 1;
+            });
             if (threadIdx.x == 0) *uv.counter() = 0;
         }
         __syncthreads();
@@ -214,15 +202,13 @@ ms_hv_kernel(const MsUnit *__restrict__ units, const uint32_t *__restrict__ tile
                 if (ok) epi_row<V, B, true>(ep, s_inv_s, s_c_prev, x, y, t[0], jsum4 - dsum[0], acc[0], apart);
             }
         }
-        if (tile_publish<V, B>(apart, uv.partials(), k, uv.counter(), U.n_tiles) && threadIdx.x < 32) {
-            ChainState *st = uv.st();
-            for (int r = 0; r < B; ++r) {
-                const double v = tile_total<B>(uv.partials(), U.n_tiles, r);
-                if (threadIdx.x == 0 && !st[r].stopped) {
-                    st[r].alpha = v;
-                    alpha[(size_t)(U.chain_base + r) * M + (ju - 1)] = v;
-                }
-            }
+        if (tile_publish<V, B>(apart, uv.partials(), k, uv.counter(), U.n_tiles)) {
+            totals<B, kRowThreads>(uv.partials(), U.n_tiles, [&](int r, double v) {
+                ChainState &c = uv.st()[r];
+                if (c.stopped) return;
+                c.alpha = v;
+                alpha[(size_t)(U.chain_base + r) * M + (ju - 1)] = v;
+            });
             if (threadIdx.x == 0) *uv.counter() = 0;
         }
         __syncthreads();
@@ -307,27 +293,25 @@ ms_update_kernel(const MsUnit *__restrict__ units, const uint32_t *__restrict__ 
             y[e] = w;
             acc[0].add(w, w);
         }
-        if (tile_publish<V, B>(acc, uv.partials(), k, uv.counter(), U.n_stiles) && threadIdx.x < 32) {
-            ChainState *st = uv.st();
-            for (int r = 0; r < B; ++r) {
-                const double bt = sqrt(tile_total<B>(uv.partials(), U.n_stiles, r));
-                if (threadIdx.x == 0 && !st[r].stopped) {
-                    ChainState &c = st[r];
-                    if (ju < U.m_max) {
-                        if (bt <= U.tau) {
-                            c.stopped = 1;
-                            c.m_eff = ju;
-                        } else {
-                            beta[(size_t)(U.chain_base + r) * M + (ju - 1)] = bt;
-                            c.s_prev = c.s_cur;
-                            c.s_cur = bt;
-                            c.beta_prev = bt;
-                        }
+        if (tile_publish<V, B>(acc, uv.partials(), k, uv.counter(), U.n_stiles)) {
+            totals<B, kRowThreads>(uv.partials(), U.n_stiles, [&](int r, double sum) {
+                ChainState &c = uv.st()[r];
+                if (c.stopped) return;
+                const double bt = sqrt(sum);
+                if (ju < U.m_max) {
+                    if (bt <= U.tau) {
+                        c.stopped = 1;
+                        c.m_eff = ju;
                     } else {
-                        c.m_eff = U.m_max;
+                        beta[(size_t)(U.chain_base + r) * M + (ju - 1)] = bt;
+                        c.s_prev = c.s_cur;
+                        c.s_cur = bt;
+                        c.beta_prev = bt;
                     }
+                } else {
+                    c.m_eff = U.m_max;
                 }
-            }
+            });
             if (threadIdx.x == 0) *uv.counter() = 0;
         }
         __syncthreads();

@@ -1,10 +1,10 @@
 // Deterministic FP64 reductions for the row-parallel kernels.
 //
-// Each block reduces its per-thread partial sums in a fixed tree (warp shuffle,
-// then one warp over the per-warp sums) and stores one partial per block.  The
-// last block to finish -- found with a fence and an atomic ticket, no waiting --
-// adds the per-block partials in index order and publishes the total.  For a
-// fixed grid the summation order never changes, so results are bit-reproducible.
+// Each block reduces its per-thread partial sums in a fixed tree (warp shuffles, then
+// the per-warp sums in order) and stores one partial per block and chain.  The last
+// block to finish -- found with a fence and an atomic ticket, no waiting -- adds the
+// per-block partials in a fixed order, one warp per chain, and publishes the totals.
+// For a fixed grid the summation order never changes, so results are bit-reproducible.
 #pragma once
 
 #include "ftlm_internal.cuh"
@@ -34,30 +34,6 @@ __device__ __forceinline__ double block_sum(double v)
     }
     __syncthreads();
     return r;
-}
-
-// Publish this block's partial; returns true (in every thread) in the last block
-// of the grid to arrive.
-__device__ __forceinline__ bool publish_partial(double part, double *partials, unsigned int *counter)
-{
-    __shared__ bool last;
-    if (threadIdx.x == 0) {
-        partials[blockIdx.x] = part;
-        __threadfence();
-        unsigned int ticket = atomicAdd(counter, 1u);
-        last = (ticket == gridDim.x - 1);
-    }
-    __syncthreads();
-    return last;
-}
-
-// Fixed-order total of partials[0 .. n-1]; call from warp 0, valid in lane 0.
-__device__ __forceinline__ double total_of_partials(const double *partials, int n)
-{
-    const int lane = threadIdx.x & 31;
-    double v = 0.0;
-    for (int i = lane; i < n; i += 32) v += __ldcg(partials + i);
-    return warp_sum(v);
 }
 
 }  // namespace ftlm
@@ -155,6 +131,62 @@ template <int B> __device__ __forceinline__ int warp_multi_index(unsigned lane)
 #pragma unroll
     for (int lvl = 0; (B >> lvl) > 1; ++lvl) r += ((lane >> lvl) & 1u) ? (B >> (lvl + 1)) : 0;
     return r;
+}
+
+// Block sums of B accumulators, in FP64: one transposed warp tree for all of them, then
+// thread r < B adds accumulator r's warp sums in warp order and returns the total
+// (other threads: 0).  Two barriers, whatever B: one tree per accumulator, each with
+// two barriers, cost 8 times the latency and the FP64 instructions at B = 8.
+template <typename V, int B, int THREADS>
+__device__ __forceinline__ double block_sums(const DotAcc<V> (&a)[B])
+{
+    constexpr int kWarps = THREADS / 32;
+    __shared__ double s_w[kWarps][B];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    DotAcc<double> p[B];
+#pragma unroll
+    for (int r = 0; r < B; ++r) p[r].v = a[r].value();
+    const DotAcc<double> t = warp_sum_multi<double, B>(p);
+    if (lane < B) s_w[wid][warp_multi_index<B>(lane)] = t.v;
+    __syncthreads();
+    double v = 0.0;
+    if (threadIdx.x < B) {
+#pragma unroll
+        for (int i = 0; i < kWarps; ++i) v += s_w[i][threadIdx.x];
+    }
+    __syncthreads();
+    return v;
+}
+
+// Stores this block's B sums (thread r < B holds the r-th) in its slot of partials;
+// returns true (in every thread) in the last block of the grid to arrive.
+template <int B>
+__device__ __forceinline__ bool publish_sums(double v, double *partials, unsigned int *counter)
+{
+    __shared__ bool s_last;
+    if (threadIdx.x < B) {
+        partials[(size_t)blockIdx.x * B + threadIdx.x] = v;
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    __syncthreads();
+    return s_last;
+}
+
+// Fixed-order totals of partials[0 .. n-1][B], one warp per accumulator, all warps at
+// once; done(r, total) runs in lane 0 of the warp that added accumulator r.
+template <int B, int THREADS, typename Done>
+__device__ __forceinline__ void totals(const double *partials, uint32_t n, Done &&done)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    for (int r = threadIdx.x >> 5; r < B; r += THREADS / 32) {
+        double v = 0.0;
+#pragma unroll 4
+        for (uint32_t g = lane; g < n; g += 32) v += __ldcg(partials + (size_t)g * B + r);
+        v = warp_sum(v);
+        if (lane == 0) done(r, v);
+    }
 }
 
 }  // namespace ftlm

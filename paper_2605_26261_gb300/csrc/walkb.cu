@@ -1,6 +1,6 @@
 // Walk B of the split Lanczos H.v (CR, spin 1/2): the high-high bonds of Eq. 12-14
 // in the transposed row order, added to walk A's output, with the Lanczos epilogue
-// (alpha as per-tile sums).  The layout of the walk is described with HiWalk in
+// (alpha from per-tile sums).  The layout of the walk is described with HiWalk in
 // ftlm_internal.cuh.
 //
 // A warp owns a tile: 32 consecutive low ranks r_lo (lane = column) of one low
@@ -57,7 +57,9 @@ walk_b_kernel(const uint32_t *__restrict__ thi, const HiWalk w, const V *__restr
     __shared__ V s_inv_s[B], s_c_prev[B];
     __shared__ uint32_t s_tile0[kMaxHiGroups + 1], s_nl[kMaxHiGroups], s_nh[kMaxHiGroups],
         s_hoff[kMaxHiGroups], s_nr[kMaxHiGroups];
+    __shared__ AlphaSums<B, walk_b_threads<V, B>()> s_asum;
     if (epi_begin<V, B>(ep, s_inv_s, s_c_prev)) return;
+    tiles_begin(s_asum);
     // group tables into shared memory (a kernel-parameter array indexed at run time
     // would be copied to local memory)
     if (threadIdx.x <= (unsigned)w.ngroups) s_tile0[threadIdx.x] = w.tile0[threadIdx.x];
@@ -166,10 +168,10 @@ walk_b_kernel(const uint32_t *__restrict__ thi, const HiWalk w, const V *__restr
                 st_vec<B>(y + t * B, out);
             }
         }
-        store_tile<V, B>(ep, tile, tacc);
+        add_tile<V, B>(ep, s_asum, tacc);
         tile = claimed_tile(claim, nwarps);
     }
-    tiles_done(ep, nwarps);
+    tiles_done(ep, s_asum);
 }
 
 template <typename V, int B, int C>
