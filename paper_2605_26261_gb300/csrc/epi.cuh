@@ -22,6 +22,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "ftlm_internal.cuh"
 #include "reduce.cuh"
@@ -37,9 +38,29 @@ struct EpiDev {
     unsigned long long *fixed;  // sums of the dynamic tile order, two words per chain
     double scale[2], unscale[2];  // 2^alpha_shift and 2^-alpha_shift as products of two factors:
                                   // the first word of a sum counts 2^-alpha_shift
+    uint64_t slot;              // bytes between the blocks of chains of a launch (blockIdx.y)
     int alpha_stride;
     int has_prev;
 };
+
+// The epilogue and the vectors of this CTA's block of chains.
+template <int B> __device__ __forceinline__ EpiDev epi_block(EpiDev ep)
+{
+    if (blockIdx.y) {
+        const uint64_t o = blockIdx.y * ep.slot;
+        ep.st = reinterpret_cast<ChainState *>(reinterpret_cast<char *>(ep.st) + o);
+        ep.partials = reinterpret_cast<double *>(reinterpret_cast<char *>(ep.partials) + o);
+        ep.counter = reinterpret_cast<unsigned int *>(reinterpret_cast<char *>(ep.counter) + o);
+        ep.fixed = reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(ep.fixed) + o);
+        ep.alpha_out += (size_t)blockIdx.y * B * ep.alpha_stride;
+    }
+    return ep;
+}
+template <typename T> __device__ __forceinline__ T *block_ptr(T *p, uint64_t slot)
+{
+    using C = typename std::conditional<std::is_const<T>::value, const char, char>::type;
+    return reinterpret_cast<T *>(reinterpret_cast<C *>(p) + blockIdx.y * slot);
+}
 
 inline EpiDev epi_of(const LanczosHv *epi)
 {
@@ -58,6 +79,7 @@ inline EpiDev epi_of(const LanczosHv *epi)
         ep.unscale[0] = 1.0 / ep.scale[0];
         ep.unscale[1] = 1.0 / ep.scale[1];
         ep.alpha_stride = epi->alpha_stride;
+        ep.slot = epi->slot;
         ep.has_prev = epi->j > 1;
     }
     return ep;

@@ -256,6 +256,8 @@ struct LanczosHv {
     int j;
     unsigned long long *fixed;  // kAlphaFixedBytes, zero between launches: alpha sums of a dynamic tile order
     double norm_bound;     // upper bound of ||H||
+    int blocks;            // blocks of B chains in the launch (>= 1), and the bytes between their vectors,
+    uint64_t slot;         // states, partials, counters and sums; alpha_out rows follow one another
 };
 // Two words per chain of a block (epi.cuh).
 constexpr uint64_t kAlphaFixedBytes = 2 * kMaxBlock * sizeof(unsigned long long);
@@ -274,6 +276,8 @@ void launch_hs_fill(const ftlm_basis *b, cudaStream_t stream);
 ftlm_status launch_hv(const ftlm_basis *b, ftlm_dtype dtype, int B, const void *x, void *y,
                       const LanczosHv *epi, cudaStream_t stream);
 bool valid_block(int B);
+// Whether a Lanczos H.v of blocks of B vectors runs as two walks (one block per launch).
+bool hv_splits(const ftlm_basis *b, ftlm_dtype dtype, int B);
 // FTLM_RANK_AUTO picks CR for sectors of at least this many rows.
 constexpr uint64_t kAutoCrRows = 1ull << 20;
 // Upper bound on the tiles of a Lanczos H.v launch of B vectors that takes its tiles

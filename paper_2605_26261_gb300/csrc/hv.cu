@@ -81,9 +81,12 @@ enum { kPlain = 0, kLanczos = 1 };
 
 template <typename V, typename Lbl, bool CLT, int EPI, int RT, int B, int C>
 __global__ void __launch_bounds__(kRowThreads, min_ctas<V, RT, B, C>())
-hv_kernel(const SectorTables s, const BondList bl, const V *__restrict__ x, V *y, const EpiDev ep)
+hv_kernel(const SectorTables s, const BondList bl, const V *__restrict__ x0, V *y0, const EpiDev ep0)
 {
     constexpr bool LANCZOS = EPI != kPlain;
+    const EpiDev ep = LANCZOS ? epi_block<B>(ep0) : ep0;
+    const V *__restrict__ x = LANCZOS ? block_ptr(x0, ep0.slot) : x0;
+    V *y = LANCZOS ? block_ptr(y0, ep0.slot) : y0;
     // CR Lanczos launches take their tiles in dynamic order (their gathers gain the
     // most from a narrow frontier of rows) and add their alpha sums per tile
     constexpr bool TILES = LANCZOS && !CLT;
@@ -149,8 +152,9 @@ hv_kernel(const SectorTables s, const BondList bl, const V *__restrict__ x, V *y
 }
 
 // alpha_j of a dynamically ordered launch from its sums (epi.cuh); one warp.
-template <int B> __global__ void __launch_bounds__(32) alpha_kernel(const EpiDev ep)
+template <int B> __global__ void __launch_bounds__(32) alpha_kernel(const EpiDev ep0)
 {
+    const EpiDev ep = epi_block<B>(ep0);
     const int r = threadIdx.x;
     if (r < B) {
         const long long hi = (long long)ep.fixed[2 * r], lo = (long long)ep.fixed[2 * r + 1];
@@ -231,7 +235,7 @@ bool split_walks(const ftlm_basis *b, int B, size_t vsize, HiWalk *w)
 
 // One hv_kernel launch over every row.
 template <typename V, typename Lbl, bool CLT, int EPI, int RT, int B, int C>
-ftlm_status launch_rows(const ftlm_basis *b, const BondList &bl, const V *x, V *y, const EpiDev &ep,
+ftlm_status launch_rows(const ftlm_basis *b, const BondList &bl, const V *x, V *y, const EpiDev &ep, int blocks,
                         cudaStream_t stream)
 {
     const size_t smem = CLT ? 0 : ((size_t)1 << b->L) * sizeof(uint16_t);
@@ -240,36 +244,36 @@ ftlm_status launch_rows(const ftlm_basis *b, const BondList &bl, const V *x, V *
     const size_t smem_max = CLT ? 0 : ((size_t)1 << kLoBitsMax) * sizeof(uint16_t);
     FTLM_CUDA(kernel_occupancy((const void *)kern, kRowThreads, smem_max, false, &occ));
     const int grid = row_grid(b, (b->D + RT - 1) / RT, std::min(occ, hv_cta_cap()));
-    kern<<<grid, kRowThreads, smem, stream>>>(b->tables(), bl, x, y, ep);
+    kern<<<dim3(grid, blocks), kRowThreads, smem, stream>>>(b->tables(), bl, x, y, ep);
     note_launch();
     return FTLM_OK;
 }
 
 template <typename V, typename Lbl, bool CLT, bool LANCZOS, int RT, int B, int C>
-ftlm_status launch(const ftlm_basis *b, const V *x, V *y, const EpiDev &ep, cudaStream_t stream)
+ftlm_status launch(const ftlm_basis *b, const V *x, V *y, const EpiDev &ep, int blocks, cudaStream_t stream)
 {
-    void *tok = profile_begin(kProfHv, stream, B);
+    void *tok = profile_begin(kProfHv, stream, B * blocks);
     ftlm_status st = FTLM_OK;
     if constexpr (LANCZOS && !CLT) {
         // CR Lanczos step: one walk over the rows, or the split (walk A, then walk B
         // over the high-high bonds in the transposed order)
         HiWalk w;
-        if (split_walks(b, B, sizeof(V), &w)) {
+        if (blocks == 1 && split_walks(b, B, sizeof(V), &w)) {
             const ftlm_dtype dt = sizeof(V) == 4 ? FTLM_F32 : FTLM_F64;
             LoWalk la;
             st = build_lo_walk(b, &la) ? launch_walk_a(b, la, dt, B, x, y, ep, stream)
                                        : fail(FTLM_EUNSUPPORTED, "split H.v without a walk A tile table");
             if (st == FTLM_OK) st = launch_walk_b(b, w, dt, B, x, y, ep, stream);
         } else {
-            st = launch_rows<V, Lbl, false, kLanczos, RT, B, C>(b, b->bonds_cr, x, y, ep, stream);
+            st = launch_rows<V, Lbl, false, kLanczos, RT, B, C>(b, b->bonds_cr, x, y, ep, blocks, stream);
         }
         if (st == FTLM_OK) {
-            alpha_kernel<B><<<1, 32, 0, stream>>>(ep);
+            alpha_kernel<B><<<dim3(1, blocks), 32, 0, stream>>>(ep);
             note_launch();
         }
     } else {
         st = launch_rows<V, Lbl, CLT, LANCZOS ? kLanczos : kPlain, RT, B, C>(b, CLT ? b->bonds_clt : b->bonds_cr, x,
-                                                                           y, ep, stream);
+                                                                           y, ep, blocks, stream);
     }
     profile_end(tok, stream);
     if (st != FTLM_OK) return st;
@@ -291,35 +295,36 @@ int chunk8()
 }
 
 template <typename V, typename Lbl, bool CLT, bool LANCZOS>
-ftlm_status launch_b(const ftlm_basis *b, int B, const void *x, void *y, const EpiDev &ep, cudaStream_t stream)
+ftlm_status launch_b(const ftlm_basis *b, int B, const void *x, void *y, const EpiDev &ep, int blocks,
+                     cudaStream_t stream)
 {
     const V *xv = (const V *)x;
     V *yv = (V *)y;
     switch (B) {
-    case 4: return launch<V, Lbl, CLT, LANCZOS, 1, 4, 8>(b, xv, yv, ep, stream);
+    case 4: return launch<V, Lbl, CLT, LANCZOS, 1, 4, 8>(b, xv, yv, ep, blocks, stream);
     case 8:
         switch (chunk8()) {
-        case 8: return launch<V, Lbl, CLT, LANCZOS, 1, 8, 8>(b, xv, yv, ep, stream);
-        case 2: return launch<V, Lbl, CLT, LANCZOS, 1, 8, 2>(b, xv, yv, ep, stream);
-        default: return launch<V, Lbl, CLT, LANCZOS, 1, 8, 4>(b, xv, yv, ep, stream);
+        case 8: return launch<V, Lbl, CLT, LANCZOS, 1, 8, 8>(b, xv, yv, ep, blocks, stream);
+        case 2: return launch<V, Lbl, CLT, LANCZOS, 1, 8, 2>(b, xv, yv, ep, blocks, stream);
+        default: return launch<V, Lbl, CLT, LANCZOS, 1, 8, 4>(b, xv, yv, ep, blocks, stream);
         }
-    case 16: return launch<V, Lbl, CLT, LANCZOS, 1, 16, 4>(b, xv, yv, ep, stream);
+    case 16: return launch<V, Lbl, CLT, LANCZOS, 1, 16, 4>(b, xv, yv, ep, blocks, stream);
     default: break;
     }
     switch (rows_per_thread(CLT)) {
-    case 1: return launch<V, Lbl, CLT, LANCZOS, 1, 1, 8>(b, xv, yv, ep, stream);
-    case 4: return launch<V, Lbl, CLT, LANCZOS, 4, 1, 8>(b, xv, yv, ep, stream);
-    default: return launch<V, Lbl, CLT, LANCZOS, 2, 1, 8>(b, xv, yv, ep, stream);
+    case 1: return launch<V, Lbl, CLT, LANCZOS, 1, 1, 8>(b, xv, yv, ep, blocks, stream);
+    case 4: return launch<V, Lbl, CLT, LANCZOS, 4, 1, 8>(b, xv, yv, ep, blocks, stream);
+    default: return launch<V, Lbl, CLT, LANCZOS, 2, 1, 8>(b, xv, yv, ep, blocks, stream);
     }
 }
 
 template <typename V, bool LANCZOS>
-ftlm_status launch_mode(const ftlm_basis *b, int B, const void *x, void *y, const EpiDev &ep,
+ftlm_status launch_mode(const ftlm_basis *b, int B, const void *x, void *y, const EpiDev &ep, int blocks,
                         cudaStream_t stream)
 {
-    if (b->mode == FTLM_RANK_CLT) return launch_b<V, uint32_t, true, LANCZOS>(b, B, x, y, ep, stream);
-    if (b->N <= 32) return launch_b<V, uint32_t, false, LANCZOS>(b, B, x, y, ep, stream);
-    return launch_b<V, uint64_t, false, LANCZOS>(b, B, x, y, ep, stream);
+    if (b->mode == FTLM_RANK_CLT) return launch_b<V, uint32_t, true, LANCZOS>(b, B, x, y, ep, blocks, stream);
+    if (b->N <= 32) return launch_b<V, uint32_t, false, LANCZOS>(b, B, x, y, ep, blocks, stream);
+    return launch_b<V, uint64_t, false, LANCZOS>(b, B, x, y, ep, blocks, stream);
 }
 
 template <typename V>
@@ -327,13 +332,19 @@ ftlm_status launch_typed(const ftlm_basis *b, int B, const void *x, void *y, con
                          cudaStream_t stream)
 {
     const EpiDev ep = epi_of(epi);
-    if (epi) return launch_mode<V, true>(b, B, x, y, ep, stream);
-    return launch_mode<V, false>(b, B, x, y, ep, stream);
+    if (epi) return launch_mode<V, true>(b, B, x, y, ep, epi->blocks, stream);
+    return launch_mode<V, false>(b, B, x, y, ep, 1, stream);
 }
 
 }  // namespace
 
 bool valid_block(int B) { return B == 1 || B == 4 || B == 8 || B == 16; }
+
+bool hv_splits(const ftlm_basis *b, ftlm_dtype dtype, int B)
+{
+    HiWalk w;
+    return b->two_s == 1 && b->mode == FTLM_RANK_CR && split_walks(b, B, dtype == FTLM_F32 ? 4 : 8, &w);
+}
 
 uint32_t hv_lanczos_tiles(const ftlm_basis *b, int B)
 {
@@ -377,10 +388,7 @@ extern "C" ftlm_status ftlm_basis_hv_schedule(const ftlm_basis *b, int B, ftlm_d
     if (!b || !used) return ftlm::fail(FTLM_EINVAL, "NULL argument");
     if (!ftlm::valid_block(B)) return ftlm::fail(FTLM_EINVAL, "block width must be 1, 4, 8 or 16");
     if (dtype != FTLM_F32 && dtype != FTLM_F64) return ftlm::fail(FTLM_EINVAL, "bad dtype");
-    ftlm::HiWalk w;
-    const bool split = b->two_s == 1 && b->mode == FTLM_RANK_CR &&
-                       ftlm::split_walks(b, B, dtype == FTLM_F32 ? 4 : 8, &w);
-    *used = split ? FTLM_HV_SPLIT : FTLM_HV_ONE_WALK;
+    *used = ftlm::hv_splits(b, dtype, B) ? FTLM_HV_SPLIT : FTLM_HV_ONE_WALK;
     return FTLM_OK;
 }
 

@@ -22,6 +22,7 @@
 
 #include <cuda.h>
 
+#include "epi.cuh"
 #include "ftlm_internal.cuh"
 #include "reduce.cuh"
 #include "vec.cuh"
@@ -33,8 +34,16 @@ namespace ftlm {
 
 namespace {
 
-struct Keys {
-    uint64_t k[kMaxBlock];
+// The blocks of chains of a launch (blockIdx.y): bytes between their vectors, states,
+// partials and counters; block k holds the chains that follow block k - 1's.
+struct BlockSlots {
+    uint64_t bytes;
+};
+
+// Keys of the start vectors: chain r of block k is keyed chain0 + k B + r.
+struct KeySpec {
+    uint64_t seed;
+    int key_n, K, chain0;
 };
 
 // Start vectors of a block of B chains (generated, or copied from src rows of
@@ -42,16 +51,26 @@ struct Keys {
 // entries.
 template <typename V, int B>
 __global__ void __launch_bounds__(kRowThreads)
-start_kernel(uint32_t D, const Keys keys, int dist, const double *__restrict__ src, V *__restrict__ u,
-             ChainState *st, double *partials, unsigned int *counter)
+start_kernel(uint32_t D, const KeySpec keys, int dist, const double *__restrict__ src, V *__restrict__ u,
+             ChainState *st, double *partials, unsigned int *counter, const BlockSlots slots)
 {
+    u = block_ptr(u, slots.bytes);
+    st = block_ptr(st, slots.bytes);
+    partials = block_ptr(partials, slots.bytes);
+    counter = block_ptr(counter, slots.bytes);
+    if (src) src += (size_t)blockIdx.y * B * D;
+    __shared__ uint64_t s_key[B];
+    if (threadIdx.x < B)
+        s_key[threadIdx.x] =
+            chain_key(keys.seed, keys.key_n, keys.K, (uint32_t)keys.chain0 + blockIdx.y * B + threadIdx.x);
+    __syncthreads();
     DotAcc<V> acc[B];
     const uint32_t stride = gridDim.x * blockDim.x;
     for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < D; t += stride) {
         V out[B];
 #pragma unroll
         for (int r = 0; r < B; ++r) {
-            const double v = src ? src[(size_t)r * D + t] : start_value(keys.k[r], t, dist);
+            const double v = src ? src[(size_t)r * D + t] : start_value(s_key[r], t, dist);
             out[r] = (V)v;
             acc[r].add(out[r], out[r]);
         }
@@ -79,8 +98,15 @@ start_kernel(uint32_t D, const Keys keys, int dist, const double *__restrict__ s
 template <typename V, int B>
 __global__ void __launch_bounds__(kRowThreads)
 update_kernel(uint32_t D, V *__restrict__ y, const V *__restrict__ u, ChainState *st, double *partials,
-              unsigned int *counter, int j, int m_max, double tau, double *beta_out, int beta_stride)
+              unsigned int *counter, int j, int m_max, double tau, double *beta_out, int beta_stride,
+              const BlockSlots slots)
 {
+    y = block_ptr(y, slots.bytes);
+    u = block_ptr(u, slots.bytes);
+    st = block_ptr(st, slots.bytes);
+    partials = block_ptr(partials, slots.bytes);
+    counter = block_ptr(counter, slots.bytes);
+    beta_out += (size_t)blockIdx.y * B * beta_stride;
     // the per-chain scalars once per CTA: a division in every thread is 10 FP64
     // instructions per chain on a pipe of two lanes per cycle (40 us per launch at B = 8,
     // whatever D)
@@ -149,9 +175,9 @@ update_kernel(uint32_t D, V *__restrict__ y, const V *__restrict__ u, ChainState
     }
 }
 
-__global__ void copy_meff_kernel(const ChainState *st, int B, int *dst)
+__global__ void copy_meff_kernel(const ChainState *st, int B, int *dst, const BlockSlots slots)
 {
-    if (threadIdx.x < B) dst[threadIdx.x] = st[threadIdx.x].m_eff;
+    if (threadIdx.x < B) dst[blockIdx.y * B + threadIdx.x] = block_ptr(st, slots.bytes)[threadIdx.x].m_eff;
 }
 
 constexpr int kRitzThreads = 128;
@@ -405,39 +431,62 @@ std::vector<int> block_plan(int R, ftlm_dtype dtype, int bmax)
     return plan;
 }
 
+// Blocks of one width that run side by side in the same launches (block k in grid row
+// y = k) while their slots fit kSideBySideBytes.  A small sector's launch is bound by
+// its dependent chain of latencies, not by the work of one block, and holds a part of
+// the SMs only: the N = 16 ring in FP64, R = 20 (five blocks of 4, 12 870 rows), takes
+// 29 us per step for all five against 5 x 28 us one after another.  At 24 MiB the rows of
+// one block of 8 floats number 0.19 million or more, enough for every SM.  A block's
+// grid and sums are those of a launch of its own, so its results do not change.
+constexpr uint64_t kSideBySideBytes = 24ull << 20;
+
+// Workspace: `slots` block slots (two vector blocks, partials, states and counters, and
+// the alpha sums of dynamically ordered H.v launches, of which kAlphaFixedBytes are
+// used), then the coefficients of every chain.
 struct Layout {
-    int bw;  // widest block
-    uint64_t vec0, vec1, partials, state, alpha, beta, meff, tiles, total;
+    int bw;     // widest block
+    int slots;  // blocks side by side
+    uint64_t slot, vec1, partials, state, tiles;  // bytes of a slot and offsets in it (vectors first)
+    uint64_t alpha, beta, meff, total;
 };
 
 Layout layout(const ftlm_basis *b, int R, int M, ftlm_dtype dtype, int bmax = 0)
 {
     Layout l;
     l.bw = 1;
-    for (int w : block_plan(R, dtype, bmax)) l.bw = w > l.bw ? w : l.bw;
+    int same = 1, most = 1, last = 0;
+    for (int w : block_plan(R, dtype, bmax)) {
+        l.bw = w > l.bw ? w : l.bw;
+        same = w == last ? same + 1 : 1;
+        last = w;
+        most = std::max(most, same);
+    }
     const uint64_t vb = align256(b->D * (uint64_t)l.bw * (dtype == FTLM_F32 ? 4ull : 8ull));
-    l.vec0 = 0;
     l.vec1 = vb;
     l.partials = 2 * vb;
     l.state = l.partials + align256((uint64_t)max_row_grid(b) * l.bw * sizeof(double));
-    l.alpha = l.state + align256(l.bw * sizeof(ChainState) + 64);
+    l.tiles = l.state + align256(l.bw * sizeof(ChainState) + 64);
+    l.slot = l.tiles + align256((uint64_t)hv_lanczos_tiles(b, 4) * l.bw * sizeof(double));
+    const uint64_t rows = 2 * align256((uint64_t)R * M * sizeof(double)) + align256((uint64_t)R * sizeof(int));
+    const uint64_t room = kSideBySideBytes > rows ? kSideBySideBytes - rows : 0;
+    l.slots = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)most, room / l.slot));
+    l.alpha = l.slots * l.slot;
     l.beta = l.alpha + align256((uint64_t)R * M * sizeof(double));
     l.meff = l.beta + align256((uint64_t)R * M * sizeof(double));
-    l.tiles = l.meff + align256((uint64_t)R * sizeof(int));
-    // alpha sums of dynamically ordered H.v launches (kAlphaFixedBytes of it are used)
-    l.total = l.tiles + align256((uint64_t)hv_lanczos_tiles(b, 4) * l.bw * sizeof(double));
+    l.total = l.meff + align256((uint64_t)R * sizeof(int));
     return l;
 }
 
-// One block of B chains: start vectors, then min(M, D) fused H.v + update launches.
+// n blocks of B chains side by side: start vectors, then min(M, D) fused H.v + update
+// launches.
 template <typename V, int B>
-ftlm_status run_block(const ftlm_basis *b, int M, int r0, int chain0, uint64_t seed, int dist, const double *src,
-                      ftlm_dtype dtype, char *ws, const Layout &lay, cudaStream_t stream)
+ftlm_status run_blocks(const ftlm_basis *b, int M, int r0, int n, int chain0, uint64_t seed, int dist,
+                       const double *src, ftlm_dtype dtype, char *ws, const Layout &lay, cudaStream_t stream)
 {
     int occ_start = 1, occ_upd = 1;
     FTLM_CUDA(kernel_occupancy((const void *)start_kernel<V, B>, kRowThreads, 0, false, &occ_start));
     FTLM_CUDA(kernel_occupancy((const void *)update_kernel<V, B>, kRowThreads, 0, false, &occ_upd));
-    V *vec[2] = {(V *)(ws + lay.vec0), (V *)(ws + lay.vec1)};
+    V *vec[2] = {(V *)ws, (V *)(ws + lay.vec1)};
     double *partials = (double *)(ws + lay.partials);
     ChainState *st = (ChainState *)(ws + lay.state);
     unsigned int *counter = (unsigned int *)(st + lay.bw);
@@ -449,32 +498,34 @@ ftlm_status run_block(const ftlm_basis *b, int M, int r0, int chain0, uint64_t s
     const double tau = dtype == FTLM_F32 ? b->tau32 : b->tau64;
     constexpr int W = 16 / (int)sizeof(V);
     constexpr int U = B > W ? B : W;
-    const int g_start = row_grid(b, D, occ_start);
-    const int g_upd = row_grid(b, ((uint64_t)D * B + U - 1) / U, occ_upd);
+    const dim3 g_start(row_grid(b, D, occ_start), n);
+    const dim3 g_upd(row_grid(b, ((uint64_t)D * B + U - 1) / U, occ_upd), n);
+    const BlockSlots slots{lay.slot};
 
-    FTLM_CUDA(cudaMemsetAsync(st, 0, lay.bw * sizeof(ChainState) + 64, stream));
-    if (lay.total > lay.tiles) FTLM_CUDA(cudaMemsetAsync(ws + lay.tiles, 0, kAlphaFixedBytes, stream));
-    Keys keys{};
-    for (int r = 0; r < B; ++r) keys.k[r] = chain_key(seed, b->key_n, b->K, (uint32_t)(chain0 + r0 + r));
-    start_kernel<V, B><<<g_start, kRowThreads, 0, stream>>>(D, keys, dist, src ? src + (size_t)r0 * D : nullptr,
-                                                           vec[0], st, partials, counter);
+    // states and counters, and the alpha sums behind them
+    const uint64_t zero = lay.slot > lay.tiles ? lay.tiles - lay.state + kAlphaFixedBytes
+                                               : lay.bw * sizeof(ChainState) + 64;
+    FTLM_CUDA(cudaMemset2DAsync(st, lay.slot, 0, zero, n, stream));
+    start_kernel<V, B><<<g_start, kRowThreads, 0, stream>>>(
+        D, KeySpec{seed, b->key_n, b->K, chain0 + r0}, dist, src ? src + (size_t)r0 * D : nullptr, vec[0], st,
+        partials, counter, slots);
     note_launch();
     FTLM_CUDA(cudaGetLastError());
     int cur = 0;
     for (int j = 1; j <= m_max; ++j) {
         LanczosHv epi{st, partials, counter, alpha_ws + (size_t)r0 * M + (j - 1), M, j,
-                      (unsigned long long *)(ws + lay.tiles), b->tau64 * (0x1p53 / 100.0)};
+                      (unsigned long long *)(ws + lay.tiles), b->tau64 * (0x1p53 / 100.0), n, lay.slot};
         ftlm_status s = launch_hv(b, dtype, B, vec[cur], vec[1 - cur], &epi, stream);
         if (s != FTLM_OK) return s;
         void *tok = profile_begin(kProfUpdate, stream);
         update_kernel<V, B><<<g_upd, kRowThreads, 0, stream>>>(D, vec[1 - cur], vec[cur], st, partials, counter, j,
-                                                               m_max, tau, beta_ws + (size_t)r0 * M, M);
+                                                               m_max, tau, beta_ws + (size_t)r0 * M, M, slots);
         note_launch();
         profile_end(tok, stream);
         FTLM_CUDA(cudaGetLastError());
         cur = 1 - cur;
     }
-    copy_meff_kernel<<<1, 32, 0, stream>>>(st, B, meff_ws + r0);
+    copy_meff_kernel<<<dim3(1, n), 32, 0, stream>>>(st, B, meff_ws + r0, slots);
     note_launch();
     FTLM_CUDA(cudaGetLastError());
     return FTLM_OK;
@@ -490,17 +541,23 @@ ftlm_status run_chains(const ftlm_basis *b, int R, int M, int chain0, uint64_t s
     int *meff_ws = (int *)(ws + lay.meff);
     FTLM_CUDA(cudaMemsetAsync(alpha_ws, 0, (size_t)R * M * sizeof(double), stream));
     FTLM_CUDA(cudaMemsetAsync(beta_ws, 0, (size_t)R * M * sizeof(double), stream));
+    const std::vector<int> plan = block_plan(R, dtype, bmax);
     int r0 = 0;
-    for (int B : block_plan(R, dtype, bmax)) {
+    for (size_t k = 0; k < plan.size();) {
+        const int B = plan[k];
+        int n = 1;  // blocks of this width that run side by side
+        const int most = hv_splits(b, dtype, B) ? 1 : lay.slots;
+        while (n < most && k + n < plan.size() && plan[k + n] == B) ++n;
         ftlm_status s;
         switch (B) {
-        case 16: s = run_block<V, 16>(b, M, r0, chain0, seed, dist, src, dtype, ws, lay, stream); break;
-        case 8: s = run_block<V, 8>(b, M, r0, chain0, seed, dist, src, dtype, ws, lay, stream); break;
-        case 4: s = run_block<V, 4>(b, M, r0, chain0, seed, dist, src, dtype, ws, lay, stream); break;
-        default: s = run_block<V, 1>(b, M, r0, chain0, seed, dist, src, dtype, ws, lay, stream); break;
+        case 16: s = run_blocks<V, 16>(b, M, r0, n, chain0, seed, dist, src, dtype, ws, lay, stream); break;
+        case 8: s = run_blocks<V, 8>(b, M, r0, n, chain0, seed, dist, src, dtype, ws, lay, stream); break;
+        case 4: s = run_blocks<V, 4>(b, M, r0, n, chain0, seed, dist, src, dtype, ws, lay, stream); break;
+        default: s = run_blocks<V, 1>(b, M, r0, n, chain0, seed, dist, src, dtype, ws, lay, stream); break;
         }
         if (s != FTLM_OK) return s;
-        r0 += B;
+        r0 += n * B;
+        k += n;
     }
     ftlm_status s = launch_ritz(R, M, alpha_ws, beta_ws, meff_ws, theta, weight, stream);
     if (s != FTLM_OK) return s;

@@ -79,9 +79,12 @@ constexpr uint64_t kSpinSmemHigh = FTLM_SPIN_SMEM_HIGH;
 
 template <typename V, bool LANCZOS, int B, bool TS>
 __global__ void __launch_bounds__(kRowThreads, B >= 8 ? FTLM_SPIN_B8_MIN_CTAS : (sizeof(V) == 8 && B >= 4 ? 2 : 3))
-hv_spin_kernel(const SectorTables s, const SpinDev p, const V *__restrict__ x, V *y, const EpiDev ep)
+hv_spin_kernel(const SectorTables s, const SpinDev p, const V *__restrict__ x0, V *y0, const EpiDev ep0)
 {
     constexpr int C = spin_chunk<B>();
+    const EpiDev ep = LANCZOS ? epi_block<B>(ep0) : ep0;
+    const V *__restrict__ x = LANCZOS ? block_ptr(x0, ep0.slot) : x0;
+    V *y = LANCZOS ? block_ptr(y0, ep0.slot) : y0;
     extern __shared__ uint16_t s_tlo[];
     // thi after tlo, at a 16-byte boundary (tlo has at most 2^14 entries)
     uint32_t *s_thi = reinterpret_cast<uint32_t *>(s_tlo + (((size_t)s.lomask + 8) & ~(size_t)7));
@@ -157,7 +160,7 @@ int grid_of(const ftlm_basis *b, uint64_t n)
 }
 
 template <typename V, bool LANCZOS, int B>
-ftlm_status launch_spin(const ftlm_basis *b, const V *x, V *y, const EpiDev &ep, cudaStream_t stream)
+ftlm_status launch_spin(const ftlm_basis *b, const V *x, V *y, const EpiDev &ep, int blocks, cudaStream_t stream)
 {
     const bool ts = b->H <= kSpinSmemHigh;
     auto kern = ts ? hv_spin_kernel<V, LANCZOS, B, true> : hv_spin_kernel<V, LANCZOS, B, false>;
@@ -167,8 +170,8 @@ ftlm_status launch_spin(const ftlm_basis *b, const V *x, V *y, const EpiDev &ep,
     FTLM_CUDA(kernel_occupancy((const void *)kern, kRowThreads, smem_max, true, &occ));
     const size_t smem = tlo_bytes + (ts ? (size_t)b->H * sizeof(uint32_t) : 0);
     const int grid = row_grid(b, b->D, occ);
-    void *tok = profile_begin(kProfHv, stream, B);
-    kern<<<grid, kRowThreads, smem, stream>>>(b->tables(), b->spin, x, y, ep);
+    void *tok = profile_begin(kProfHv, stream, B * blocks);
+    kern<<<dim3(grid, blocks), kRowThreads, smem, stream>>>(b->tables(), b->spin, x, y, ep);
     note_launch();
     profile_end(tok, stream);
     FTLM_CUDA(cudaGetLastError());
@@ -176,16 +179,16 @@ ftlm_status launch_spin(const ftlm_basis *b, const V *x, V *y, const EpiDev &ep,
 }
 
 template <typename V, bool LANCZOS>
-ftlm_status launch_spin_b(const ftlm_basis *b, int B, const void *x, void *y, const EpiDev &ep,
+ftlm_status launch_spin_b(const ftlm_basis *b, int B, const void *x, void *y, const EpiDev &ep, int blocks,
                           cudaStream_t stream)
 {
     const V *xv = (const V *)x;
     V *yv = (V *)y;
     switch (B) {
-    case 4: return launch_spin<V, LANCZOS, 4>(b, xv, yv, ep, stream);
-    case 8: return launch_spin<V, LANCZOS, 8>(b, xv, yv, ep, stream);
-    case 16: return launch_spin<V, LANCZOS, 16>(b, xv, yv, ep, stream);
-    default: return launch_spin<V, LANCZOS, 1>(b, xv, yv, ep, stream);
+    case 4: return launch_spin<V, LANCZOS, 4>(b, xv, yv, ep, blocks, stream);
+    case 8: return launch_spin<V, LANCZOS, 8>(b, xv, yv, ep, blocks, stream);
+    case 16: return launch_spin<V, LANCZOS, 16>(b, xv, yv, ep, blocks, stream);
+    default: return launch_spin<V, LANCZOS, 1>(b, xv, yv, ep, blocks, stream);
     }
 }
 
@@ -195,11 +198,12 @@ ftlm_status launch_hv_spin(const ftlm_basis *b, ftlm_dtype dtype, int B, const v
                            const LanczosHv *epi, cudaStream_t stream)
 {
     const EpiDev ep = epi_of(epi);
+    const int n = epi ? epi->blocks : 1;
     if (dtype == FTLM_F32)
-        return epi ? launch_spin_b<float, true>(b, B, x, y, ep, stream)
-                   : launch_spin_b<float, false>(b, B, x, y, ep, stream);
-    return epi ? launch_spin_b<double, true>(b, B, x, y, ep, stream)
-               : launch_spin_b<double, false>(b, B, x, y, ep, stream);
+        return epi ? launch_spin_b<float, true>(b, B, x, y, ep, n, stream)
+                   : launch_spin_b<float, false>(b, B, x, y, ep, n, stream);
+    return epi ? launch_spin_b<double, true>(b, B, x, y, ep, n, stream)
+               : launch_spin_b<double, false>(b, B, x, y, ep, n, stream);
 }
 
 ftlm_status launch_spin_labels(const ftlm_basis *b, uint64_t first, uint64_t count, uint64_t *out,
