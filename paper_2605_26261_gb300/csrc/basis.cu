@@ -377,17 +377,14 @@ ftlm_status ftlm::basis_create_half(int N, int two_sz, int n_bonds, const int *b
     double jsum4 = 0.0;
     for (int k = 0; k < n_bonds; ++k) jsum4 += J[k] / 4.0;
     auto round_up = [](int v) { return (v + kBondChunk - 1) / kBondChunk * kBondChunk; };
-    // host images of the slot arrays: CR, CLT and walk A (FP32 and FP64 each), walk B
+    // host images of the slot arrays: CR and CLT (FP32), rows of doubles, walk A (FP32 and
+    // FP64), walk B
     std::vector<uint4> slots(7 * (size_t)kMaxBondSlots, make_uint4(0u, 0u, 0u, 0u));
     auto put = [&](int which, int pos, uint32_t mlo, uint32_t mhi, double jh) {
         float f = (float)jh;
         uint32_t fb;
         std::memcpy(&fb, &f, 4);
-        uint64_t db;
-        std::memcpy(&db, &jh, 8);
         slots[(size_t)(2 * which) * kMaxBondSlots + pos] = make_uint4(mlo, mhi, fb, 0u);
-        slots[(size_t)(2 * which + 1) * kMaxBondSlots + pos] =
-            make_uint4(mlo, mhi, (uint32_t)db, (uint32_t)(db >> 32));
     };
     {
         BondList &c = b->bonds_cr;
@@ -471,6 +468,31 @@ ftlm_status ftlm::basis_create_half(int N, int two_sz, int n_bonds, const int *b
         c.n_lo = c.n_hi = 0;
         c.nb = round_up(n_bonds);
         c.jsum4 = jsum4;
+    }
+    {
+        // rows of doubles: highest lower site first
+        std::vector<int> order(n_bonds);
+        for (int k = 0; k < n_bonds; ++k) order[k] = k;
+        std::stable_sort(order.begin(), order.end(), [&](int p, int q) {
+            return std::min(bi[p], bj[p]) > std::min(bi[q], bj[q]);
+        });
+        for (int pos = 0; pos < n_bonds; ++pos) {
+            const int k = order[pos];
+            const uint64_t m = (1ull << bi[k]) | (1ull << bj[k]);
+            const double jh = J[k] / 2.0;
+            uint64_t db;
+            std::memcpy(&db, &jh, 8);
+            slots[(size_t)kMaxBondSlots + pos] =
+                make_uint4((uint32_t)m, (uint32_t)(m >> 32), (uint32_t)db, (uint32_t)(db >> 32));
+        }
+        // sums of J/2 stay below 2^61 units
+        const int e = jabs > 0.0 ? std::ilogb(jabs) + 1 : 0;
+        const int shift = std::min(1000, 61 - e);
+        for (BondList *c : {&b->bonds_cr, &b->bonds_clt}) {
+            c->n64 = n_bonds;
+            c->jscale = std::ldexp(1.0, shift);
+            c->junscale = std::ldexp(1.0, -shift);
+        }
     }
 
     // Digit-block tables on the host.
@@ -591,7 +613,7 @@ ftlm_status ftlm::basis_create_half(int N, int two_sz, int n_bonds, const int *b
     b->bonds_cr.slots_f32 = b->bond_slots;
     b->bonds_cr.slots_f64 = b->bond_slots + kMaxBondSlots;
     b->bonds_clt.slots_f32 = b->bond_slots + 2 * kMaxBondSlots;
-    b->bonds_clt.slots_f64 = b->bond_slots + 3 * kMaxBondSlots;
+    b->bonds_clt.slots_f64 = b->bonds_cr.slots_f64;
 
     // The copy returns once the image is staged, so `image` may go out of scope;
     // the kernels below follow it in stream order.

@@ -119,7 +119,7 @@ batch_kernel(const BatchItemDev *__restrict__ items, const BatchUnitDev *__restr
              double *beta_all, int *meff_all)
 {
     extern __shared__ uint16_t s_tlo[];
-    __shared__ uint4 s_bond[kMaxBondSlots];
+    __shared__ RowBonds<V, Lbl> s_bond;
     __shared__ double s_warp[(kBatchThreads / 32) * B];
     __shared__ double s_tot[B], s_cur[B], s_prev[B], s_bprev[B];
     __shared__ V s_inv_s[B], s_cprev[B], s_a[B];
@@ -143,8 +143,7 @@ batch_kernel(const BatchItemDev *__restrict__ items, const BatchUnitDev *__restr
         const double tau = it.tau;
         const size_t cbase = (size_t)it.chain_base + un.r0;
         {
-            const uint4 *src = sizeof(V) == 4 ? bl.slots_f32 : bl.slots_f64;
-            for (int i = threadIdx.x; i < bl.nb; i += kBatchThreads) s_bond[i] = src[i];
+            s_bond.stage(bl);
             if (!CLT)
                 for (uint32_t i = threadIdx.x; i <= s.lomask; i += kBatchThreads) s_tlo[i] = __ldg(s.tlo + i);
         }
@@ -194,19 +193,15 @@ batch_kernel(const BatchItemDev *__restrict__ items, const BatchUnitDev *__restr
             // y = H q_j - beta_{j-1} q_{j-1} (over u_{j-1}), alpha partials
             DotAcc<V> ap[B];
             for (uint32_t t = threadIdx.x; t < D; t += kBatchThreads) {
-                const uint32_t tt[1] = {t};
-                V acc[1][B], dsum[1] = {(V)0};
-#pragma unroll
-                for (int r = 0; r < B; ++r) acc[0][r] = (V)0;
-                if (CLT) rows_clt<V, 1, B, C, false>(s, bl, s_bond, x, tt, acc, dsum);
-                else rows_cr<V, Lbl, 1, B, C, false>(s, bl, s_bond, s_tlo, x, tt, acc, dsum);
+                V acc[B], dsum;
+                row_sums<V, Lbl, CLT, B, C, false>(s, bl, s_bond, s_tlo, x, t, acc, dsum);
                 V xt[B], up[B], out[B];
                 ld_vec_coherent<B>(x + (size_t)t * B, xt);
                 if (j > 1) ld_vec_coherent<B>(y + (size_t)t * B, up);
-                const V diag = (V)bl.jsum4 - dsum[0];
+                const V diag = (V)bl.jsum4 - dsum;
 #pragma unroll
                 for (int r = 0; r < B; ++r) {
-                    const V hv = fma(diag, xt[r], acc[0][r]);
+                    const V hv = fma(diag, xt[r], acc[r]);
                     out[r] = j > 1 ? fma(-s_cprev[r], up[r], hv * s_inv_s[r]) : hv * s_inv_s[r];
                     ap[r].add(xt[r] * s_inv_s[r], out[r]);
                 }

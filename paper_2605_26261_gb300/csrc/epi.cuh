@@ -36,8 +36,8 @@ struct EpiDev {
     unsigned int *counter;  // [0] block ticket; [1], [2], [3] dynamic tile order
     double *alpha_out;
     unsigned long long *fixed;  // sums of the dynamic tile order, two words per chain
-    double scale[2], unscale[2];  // 2^alpha_shift and 2^-alpha_shift as products of two factors:
-                                  // the first word of a sum counts 2^-alpha_shift
+    double scale, unscale;      // 2^alpha_shift and 2^-alpha_shift: the first word of a sum
+                                // counts 2^-alpha_shift
     uint64_t slot;              // bytes between the blocks of chains of a launch (blockIdx.y)
     int alpha_stride;
     int has_prev;
@@ -71,13 +71,12 @@ inline EpiDev epi_of(const LanczosHv *epi)
         ep.counter = epi->counter;
         ep.alpha_out = epi->alpha_out;
         ep.fixed = epi->fixed;
-        // |alpha_j| <= ||H|| < 2^e: counting 2^-(60 - e) keeps the sum below 2^60
+        // |alpha_j| <= ||H|| < 2^e, and ||y|| <= 2 ||H||: a tile's sum stays below 2^50
+        // units, that of all tiles within 64 bits
         const int e = epi->norm_bound > 0.0 ? std::ilogb(epi->norm_bound) + 1 : 0;
-        const int shift = 60 - e;
-        ep.scale[0] = std::ldexp(1.0, shift / 2);
-        ep.scale[1] = std::ldexp(1.0, shift - shift / 2);
-        ep.unscale[0] = 1.0 / ep.scale[0];
-        ep.unscale[1] = 1.0 / ep.scale[1];
+        const int shift = std::min(1000, 49 - e);
+        ep.scale = std::ldexp(1.0, shift);
+        ep.unscale = std::ldexp(1.0, -shift);
         ep.alpha_stride = epi->alpha_stride;
         ep.slot = epi->slot;
         ep.has_prev = epi->j > 1;
@@ -181,7 +180,7 @@ __device__ __forceinline__ uint32_t claimed_tile(uint32_t claim, uint32_t nwarps
 
 // Sums of per-tile values as whole numbers of two words, one pair per warp and chain in
 // shared memory: the first word counts 2^-alpha_shift, the second 2^-(alpha_shift +
-// 40).  Every value is taken to 2^-(alpha_shift + 40), about 2^-100 ||H||, and whole
+// 40).  Every value is taken to 2^-(alpha_shift + 40), about 2^-90 ||H||, and whole
 // numbers add in any order to the same sum, so the warps may take their tiles in any
 // order.  bad: bit r is set when a value of chain r was not finite.
 template <int B, int THREADS> struct AlphaSums {
@@ -206,11 +205,14 @@ __device__ __forceinline__ void add_tile(const EpiDev &ep, AlphaSums<B, THREADS>
     if (lane < B) {
         const int r = warp_multi_index<B>(lane);
         long long *w = s.v[threadIdx.x >> 5] + 2 * r;
-        const double v = t.value() * ep.scale[0] * ep.scale[1];
-        const double h = rint(v);
-        if (!(fabs(v) < 0x1p62)) atomicOr(&s.bad, 1u << r);
-        w[0] += (long long)h;
-        w[1] += (long long)rint((v - h) * 0x1p40);
+        // whole numbers through the mantissa of 1.5 2^52 + v: four FP64 instructions
+        // (conversions to 64-bit integers and back would be four more)
+        constexpr double kOne = 0x1.8p52;
+        const double a = t.value(), m = fma(a, ep.scale, kOne), h = m - kOne;
+        const double f = fma(fma(a, ep.scale, -h), 0x1p40, kOne);
+        if (!(fabs(h) < 0x1p51)) atomicOr(&s.bad, 1u << r);
+        w[0] += __double_as_longlong(m) - __double_as_longlong(kOne);
+        w[1] += __double_as_longlong(f) - __double_as_longlong(kOne);
     }
 }
 

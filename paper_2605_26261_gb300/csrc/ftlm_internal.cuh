@@ -36,6 +36,7 @@ constexpr int kMaxBondSlots = FTLM_MAX_BONDS + 2 * kBondChunk;
 //        [n_lo + n_hi, nb) any bond (full two-bit mask = mlo | mhi << 32).
 //        n_lo and n_hi are whole chunks; bonds left over go to the last range.
 //   CLT: [0, nb) in the caller's order, full mask in mlo (N <= 32).
+// (These two orders are those of FP32 rows.)
 struct BondList {
     int nb;    // slots in use, a multiple of kBondChunk
     int n_lo;
@@ -43,7 +44,12 @@ struct BondList {
     int pad;
     double jsum4;  // sum_b J_b / 4 : the diagonal when every bond is parallel
     const uint4 *slots_f32;  // J/2 as float in .z
+    // FP64 rows (row_f64): n64 bonds with their full masks, in the order of their lower
+    // site, highest first
     const uint4 *slots_f64;  // J/2 as double in .z (low word), .w (high word)
+    int n64;
+    int pad64;
+    double jscale, junscale;  // 2^jshift and its inverse: J/2 as a whole number
 };
 
 // Scalars of one Lanczos chain, kept on the device between launches.  The stored
@@ -178,7 +184,7 @@ struct ftlm_basis {
     int n_hi_bonds;                // high-high bonds (walk B of the split H.v)
     double jsum4_hi;               // their sum of J_b / 4
     void *block;        // one pooled device allocation holding every table below
-    uint4 *bond_slots;  // device: cr f32, cr f64, clt f32, clt f64, walk-A f32, walk-A f64
+    uint4 *bond_slots;  // device: cr f32, rows of doubles, clt f32, unused, walk-A f32, walk-A f64
                         // (LoWalk layout), walk-B bonds (kMaxBondSlots each)
     uint32_t *uhi;      // CR: high patterns grouped by popcount, ascending (walk B)
     uint32_t *lo_tiles; // CR: walk A tile table of the split H.v (LoWalk), or null

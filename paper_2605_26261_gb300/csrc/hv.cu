@@ -59,9 +59,8 @@ namespace {
 // 256 threads, the shared-memory limit of the CR kernel); 4 rows per thread and
 // blocks of 4-8 vectors get at least 3 CTAs per SM (fewer starve the loads), 2 with
 // 8-bond chunks of 8-wide blocks (their 16 gathers per row in flight carry it);
-// 16-wide blocks keep all their registers (a cap spills).  FP64 vectors need about
-// twice the registers: 4 CTAs for single vectors (3 with 2 rows per thread, 2 with
-// 4), 2 for blocks of 4 and 1 for wider blocks, none of them spilling.
+// 16-wide blocks keep all their registers (a cap spills).  FP64 rows (row_f64): 3 CTAs
+// up to blocks of 4, 2 for blocks of 8 and 1 for wider ones.
 // Build option FTLM_B8_MIN_CTAS: the FP32 cut for 8-wide blocks with chunks of 4.
 #ifndef FTLM_B8_MIN_CTAS
 #define FTLM_B8_MIN_CTAS 3
@@ -69,8 +68,8 @@ namespace {
 
 template <typename V, int RT, int B, int C> __host__ __device__ constexpr int min_ctas()
 {
-    if (sizeof(V) == 8)  // FP64 accumulators and gathers take twice the registers
-        return B >= 8 ? 1 : (B >= 4 ? 2 : (RT >= 4 ? 2 : (RT >= 2 ? 3 : 4)));
+    if (sizeof(V) == 8)
+        return B >= 16 ? 1 : (B >= 8 ? 2 : 3);
     return B >= 16 ? 1
                    : (B >= 8 && C >= 8 ? 2
                                        : (B >= 8 && C <= 2 ? 4 : (B >= 8 ? FTLM_B8_MIN_CTAS : (B >= 4 || RT >= 4 ? 3 : 6))));
@@ -91,15 +90,12 @@ hv_kernel(const SectorTables s, const BondList bl, const V *__restrict__ x0, V *
     // most from a narrow frontier of rows) and add their alpha sums per tile
     constexpr bool TILES = LANCZOS && !CLT;
     extern __shared__ uint16_t s_tlo[];
-    __shared__ uint4 s_bond[kMaxBondSlots];
+    __shared__ RowBonds<V, Lbl> s_bond;
     __shared__ V s_inv_s[B], s_c_prev[B];  // per-chain scalars of the epilogue
     __shared__ AlphaSums<TILES ? B : 1, kRowThreads> s_asum;
     if (LANCZOS && epi_begin<V, B>(ep, s_inv_s, s_c_prev)) return;
     if constexpr (TILES) tiles_begin(s_asum);
-    {
-        const uint4 *src = sizeof(V) == 4 ? bl.slots_f32 : bl.slots_f64;
-        for (int i = threadIdx.x; i < bl.nb; i += blockDim.x) s_bond[i] = src[i];
-    }
+    s_bond.stage(bl);
     if (!CLT)
         for (uint32_t i = threadIdx.x; i <= s.lomask; i += blockDim.x) s_tlo[i] = __ldg(s.tlo + i);
     __syncthreads();
@@ -127,8 +123,14 @@ hv_kernel(const SectorTables s, const BondList bl, const V *__restrict__ x0, V *
 #pragma unroll
             for (int r = 0; r < B; ++r) acc[i][r] = (V)0;
         }
-        if (CLT) rows_clt<V, RT, B, C>(s, bl, s_bond, x, t, acc, dsum);
-        else rows_cr<V, Lbl, RT, B, C>(s, bl, s_bond, s_tlo, x, t, acc, dsum);
+        if constexpr (sizeof(V) == 8) {
+            static_assert(RT == 1 || sizeof(V) == 4, "one row of doubles per thread");
+            row_f64<Lbl, CLT, B, C>(s, bl, s_bond.l, s_tlo, x, t[0], acc[0], dsum[0]);
+        } else if constexpr (CLT) {
+            rows_clt<V, RT, B, C>(s, bl, s_bond.e, x, t, acc, dsum);
+        } else {
+            rows_cr<V, Lbl, RT, B, C>(s, bl, s_bond.e, s_tlo, x, t, acc, dsum);
+        }
         if constexpr (TILES) {
             DotAcc<V> tacc[B];
 #pragma unroll
@@ -159,7 +161,7 @@ template <int B> __global__ void __launch_bounds__(32) alpha_kernel(const EpiDev
     if (r < B) {
         const long long hi = (long long)ep.fixed[2 * r], lo = (long long)ep.fixed[2 * r + 1];
         const bool bad = (ep.counter[3] >> r) & 1u;
-        const double v = ((double)hi + (double)lo * 0x1p-40) * ep.unscale[0] * ep.unscale[1];
+        const double v = ((double)hi + (double)lo * 0x1p-40) * ep.unscale;
         ep.fixed[2 * r] = 0;
         ep.fixed[2 * r + 1] = 0;
         if (!ep.st[r].stopped) {
@@ -242,9 +244,17 @@ ftlm_status launch_rows(const ftlm_basis *b, const BondList &bl, const V *x, V *
     auto kern = hv_kernel<V, Lbl, CLT, EPI, RT, B, C>;
     int occ = 1;  // resident blocks per SM for this instantiation
     const size_t smem_max = CLT ? 0 : ((size_t)1 << kLoBitsMax) * sizeof(uint16_t);
-    FTLM_CUDA(kernel_occupancy((const void *)kern, kRowThreads, smem_max, false, &occ));
-    const int grid = row_grid(b, (b->D + RT - 1) / RT, std::min(occ, hv_cta_cap()));
-    kern<<<dim3(grid, blocks), kRowThreads, smem, stream>>>(b->tables(), bl, x, y, ep);
+    // A plain H.v has no block sums, so its blocks may be smaller: with the CLT (no table
+    // to stage per block) a sector too small for one block of kRowThreads rows on every
+    // SM is cut into smaller ones.
+    int threads = kRowThreads;
+    if (CLT && EPI == kPlain)
+        while (threads > 64 && b->D < (uint64_t)threads * RT * b->num_sms) threads /= 2;
+    FTLM_CUDA(kernel_occupancy((const void *)kern, threads, smem_max, false, &occ));
+    const uint64_t need = (b->D + (uint64_t)threads * RT - 1) / ((uint64_t)threads * RT);
+    const uint64_t cap = (uint64_t)b->num_sms * std::max(1, std::min({occ, hv_cta_cap(), kMaxBlocksPerSm}));
+    const int grid = (int)std::max<uint64_t>(1, std::min(need, cap));
+    kern<<<dim3(grid, blocks), threads, smem, stream>>>(b->tables(), bl, x, y, ep);
     note_launch();
     return FTLM_OK;
 }
@@ -300,6 +310,14 @@ ftlm_status launch_b(const ftlm_basis *b, int B, const void *x, void *y, const E
 {
     const V *xv = (const V *)x;
     V *yv = (V *)y;
+    if constexpr (sizeof(V) == 8) {
+        switch (B) {
+        case 4: return launch<V, Lbl, CLT, LANCZOS, 1, 4, f64_gathers<4>()>(b, xv, yv, ep, blocks, stream);
+        case 8: return launch<V, Lbl, CLT, LANCZOS, 1, 8, f64_gathers<8>()>(b, xv, yv, ep, blocks, stream);
+        case 16: return launch<V, Lbl, CLT, LANCZOS, 1, 16, f64_gathers<16>()>(b, xv, yv, ep, blocks, stream);
+        default: return launch<V, Lbl, CLT, LANCZOS, 1, 1, f64_gathers<1>()>(b, xv, yv, ep, blocks, stream);
+        }
+    } else {
     switch (B) {
     case 4: return launch<V, Lbl, CLT, LANCZOS, 1, 4, 8>(b, xv, yv, ep, blocks, stream);
     case 8:
@@ -315,6 +333,7 @@ ftlm_status launch_b(const ftlm_basis *b, int B, const void *x, void *y, const E
     case 1: return launch<V, Lbl, CLT, LANCZOS, 1, 1, 8>(b, xv, yv, ep, blocks, stream);
     case 4: return launch<V, Lbl, CLT, LANCZOS, 4, 1, 8>(b, xv, yv, ep, blocks, stream);
     default: return launch<V, Lbl, CLT, LANCZOS, 2, 1, 8>(b, xv, yv, ep, blocks, stream);
+    }
     }
 }
 
@@ -349,7 +368,7 @@ bool hv_splits(const ftlm_basis *b, ftlm_dtype dtype, int B)
 uint32_t hv_lanczos_tiles(const ftlm_basis *b, int B)
 {
     if (b->two_s > 1 || b->mode == FTLM_RANK_CLT) return 0;
-    const uint64_t rows = 32ull * (B == 1 ? rows_per_thread(false) : 1);
+    const uint64_t rows = 32ull * (B == 1 ? rows_per_thread(false) : 1);  // FP32; rows of doubles take 32
     uint32_t n = (uint32_t)((b->D + rows - 1) / rows);
     HiWalk w;  // walk B has the most tiles with one high pattern per tile
     if (build_hi_walk(b, 1, &w)) n = std::max(n, w.ntiles);

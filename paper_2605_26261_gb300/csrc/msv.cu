@@ -27,6 +27,11 @@ namespace ftlm {
 
 namespace {
 
+// The bonds of a general-spin unit in shared memory.
+struct SpinBonds {
+    uint4 e[kMaxBondSlots];
+};
+
 struct UnitView {
     const MsUnit *u;
     char *ws;
@@ -131,7 +136,7 @@ ms_hv_kernel(const MsUnit *__restrict__ units, const uint32_t *__restrict__ tile
 {
     constexpr bool CLT = KIND == kMsClt, SPIN = KIND == kMsSpin;
     extern __shared__ uint16_t s_tlo[];
-    __shared__ uint4 s_bond[kMaxBondSlots];
+    __shared__ typename std::conditional<SPIN, SpinBonds, RowBonds<V, uint32_t>>::type s_bond;
     __shared__ V s_J[SPIN ? kMaxBondSlots : 1];
     __shared__ V s_cf[SPIN ? kSpinCoef : 1];
     __shared__ V s_inv_s[B], s_c_prev[B];
@@ -151,15 +156,14 @@ ms_hv_kernel(const MsUnit *__restrict__ units, const uint32_t *__restrict__ tile
         if (ui != loaded) {  // CTA-uniform: stage the unit's bonds, tlo and chain scalars
             __syncthreads();  // every thread is past its last read of the previous unit's data
             loaded = ui;
-            if (SPIN) {
+            if constexpr (SPIN) {
                 for (uint32_t i = threadIdx.x; i < U.spin.nb; i += blockDim.x) {
-                    s_bond[i] = U.spin.slots[i];
+                    s_bond.e[i] = U.spin.slots[i];
                     s_J[i] = spin_J<V>(U.spin)[i];
                 }
                 spin_stage_coef<V>(U.spin, s_cf);
             } else {
-                const uint4 *src = sizeof(V) == 4 ? U.bl.slots_f32 : U.bl.slots_f64;
-                for (int i = threadIdx.x; i < U.bl.nb; i += blockDim.x) s_bond[i] = src[i];
+                s_bond.stage(U.bl);
             }
             if (!CLT)
                 for (uint32_t i = threadIdx.x; i <= U.s.lomask; i += blockDim.x) s_tlo[i] = __ldg(U.s.tlo + i);
@@ -188,18 +192,15 @@ ms_hv_kernel(const MsUnit *__restrict__ units, const uint32_t *__restrict__ tile
             const uint32_t tt = row0 + p + threadIdx.x;
             if (row0 + p >= D) break;  // CTA-uniform
             const bool ok = tt < D;
-            const uint32_t t[1] = {ok ? tt : D - 1};  // rows past the end recompute the last row, unstored
+            const uint32_t t = ok ? tt : D - 1;  // rows past the end recompute the last row, unstored
             if constexpr (SPIN) {
                 V acc[B], diag;
-                spin_row<V, B, C, false>(U.s, U.spin, s_tlo, nullptr, s_bond, s_J, s_cf, x, t[0], acc, diag);
-                if (ok) epi_row<V, B, true>(ep, s_inv_s, s_c_prev, x, y, t[0], diag, acc, apart);
+                spin_row<V, B, C, false>(U.s, U.spin, s_tlo, nullptr, s_bond.e, s_J, s_cf, x, t, acc, diag);
+                if (ok) epi_row<V, B, true>(ep, s_inv_s, s_c_prev, x, y, t, diag, acc, apart);
             } else {
-                V acc[1][B], dsum[1] = {(V)0};
-#pragma unroll
-                for (int r = 0; r < B; ++r) acc[0][r] = (V)0;
-                if (CLT) rows_clt<V, 1, B, C>(U.s, U.bl, s_bond, x, t, acc, dsum);
-                else rows_cr<V, uint32_t, 1, B, C>(U.s, U.bl, s_bond, s_tlo, x, t, acc, dsum);
-                if (ok) epi_row<V, B, true>(ep, s_inv_s, s_c_prev, x, y, t[0], jsum4 - dsum[0], acc[0], apart);
+                V acc[B], dsum;
+                row_sums<V, uint32_t, CLT, B, C, true>(U.s, U.bl, s_bond, s_tlo, x, t, acc, dsum);
+                if (ok) epi_row<V, B, true>(ep, s_inv_s, s_c_prev, x, y, t, jsum4 - dsum, acc, apart);
             }
         }
         if (tile_publish<V, B>(apart, uv.partials(), k, uv.counter(), U.n_tiles)) {
