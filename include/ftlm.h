@@ -329,19 +329,19 @@ ftlm_status ftlm_lanczos_noalloc(const ftlm_basis *basis, int R, int M, uint64_t
  *   first_chain + r under `seed` (the start-vector definition of ftlm_lanczos);
  *   outputs theta_dev, weight_dev (double[R*M]) and m_eff_dev (int[R]) as for
  *   ftlm_lanczos.  The basis and the outputs must outlive every run of the batch.
- * ftlm_batch_create -- plan a batch: sectors with D <= 32768 are cut into units
- *   of `block` chains (block = 1, 4, 8 or 16; 0 = 16 for FP32, 8 for FP64) that one
+ * ftlm_batch_create -- plan a batch: spin-1/2 sectors with D <= 4096 (32768 when N >
+ *   32) are cut into units of `block` chains (block = 1, 4, 8 or 16; 0 = 8) that one
  *   persistent kernel runs, one CTA per unit at a time, each unit's chains entirely
  *   inside its CTA (vectors in a per-CTA workspace slot, CTA-local reductions).
  *   Larger spin-1/2 sectors with N <= 32, and every general-spin sector, are cut
  *   into units of `block` chains that advance together, all units of a wave per
  *   launch (two launches per Lanczos step: H.v with alpha, update with beta;
  *   per-unit reductions over tiles of 2048 rows for H.v, handed out in order from
- *   a counter, and 16384 rows for the update; waves of at most FTLM_MS_WAVE_MB =
- *   256 MB of vectors) on a stream forked from the caller's.  Spin-1/2 sectors
- *   with N > 32 run the launch sequence of ftlm_lanczos with blocks of up to
- *   `block` chains, spread over up to `streams` side streams (1..8; 0 =
- *   FTLM_BATCH_STREAMS or 4).  Uploads the plan's descriptors on
+ *   a counter, and D / 32 rows, 2048 to 16384, for the update; waves of at most
+ *   FTLM_MS_WAVE_MB = 256 MB of vectors) on a stream forked from the caller's.
+ *   Larger spin-1/2 sectors with N > 32 run the launch sequence of ftlm_lanczos with
+ *   blocks of up to `block` chains, spread over up to `streams` side streams (1..8;
+ *   0 = FTLM_BATCH_STREAMS or 4).  Uploads the plan's descriptors on
  *   `stream` (one block from the library's device memory pool, owned by the
  *   batch) and returns when they are in place.  EINVAL for an empty batch or bad
  *   items.
@@ -380,7 +380,7 @@ ftlm_status ftlm_batch_destroy_async(ftlm_batch *batch, void *stream);
 /* Batch plans with explicit tile sizes.  ftlm_batch_plan: block and streams as for
  * ftlm_batch_create; tile_rows = rows per H.v tile and stream_rows = rows per tile
  * of the start/update kernels of the multi-sector path (multiples of 256 up to
- * 2^20; 0: 2048 and 16384).  ftlm_batch_create_plan plans with them (results agree
+ * 2^20; 0: 2048, and D / 32 between 2048 and 16384).  ftlm_batch_create_plan plans with them (results agree
  * with other plans up to the summation order of the per-tile sums).
  * ftlm_batch_autotune_plan times candidate plans on the items (each candidate: one
  * untimed and one timed run, as ftlm_batch_autotune) by coordinate search -- block

@@ -2,7 +2,7 @@
 //
 // A batch lists sectors (of one or many clusters) with R chains each, routed by
 // size:
-//  - spin-1/2 sectors of dimension above kSmallRows with N <= 32, and every
+//  - spin-1/2 sectors of dimension above kPersistentRows with N <= 32, and every
 //    general-spin sector, run the multi-sector path (msv.cu): units of B chains
 //    of many sectors advance together, two launches per Lanczos step per wave, on
 //    a stream forked from the caller's;
@@ -54,7 +54,15 @@ uint64_t ms_wave_bytes()
 namespace {
 
 constexpr int kBatchThreads = 256;
-constexpr uint64_t kSmallRows = 1u << 15;  // sectors up to this dimension run inside one CTA
+// Sectors up to this dimension run inside one CTA: spin-1/2 with N <= 32, and N > 32
+// (whose other path is one launch sequence per sector).  One CTA takes about 4 us per
+// 256 rows and step, a unit of the multi-sector path one tile per 2048 rows of a launch
+// that the wave runs anyway.  Measured (whole batch, every sector, FP32): clusters of 18, 17
+// and 19 sites, 16 chains x 100 steps, threshold 32768 / 16384 / 8192 / 4096 / 1024 rows:
+// 68.4 / 25.8 / 14.7 / 15.0 / 15.0 ms; 14, 15 and 16 sites, 5 x 60: 13.3 / 13.3 / 9.0 / 4.3 /
+// 4.0 ms; forty clusters of 16 sites (throughput-bound): 51.6 / 51.2 / 46.4 / 49.9 / 50.1 ms.
+constexpr uint64_t kPersistentRows = 1u << 12;
+constexpr uint64_t kSmallRows = 1u << 15;
 constexpr int kMaxSideStreams = 8;
 
 
@@ -365,7 +373,6 @@ ftlm_status batch_create(int n, const ftlm_batch_item *items, int M, ftlm_vec_di
 {
     if (!out) return fail(FTLM_EINVAL, "out is NULL");
     if (tile_rows == 0) tile_rows = kMsTileRows;
-    if (stream_rows == 0) stream_rows = kMsStreamRows;
     if (tile_rows % kRowThreads || stream_rows % kRowThreads || tile_rows > (1u << 20) || stream_rows > (1u << 20))
         return fail(FTLM_EINVAL, "tile rows must be multiples of 256 up to 2^20");
     *out = nullptr;
@@ -373,7 +380,7 @@ ftlm_status batch_create(int n, const ftlm_batch_item *items, int M, ftlm_vec_di
     if (M < 1 || M > FTLM_MAX_LANCZOS) return fail(FTLM_EINVAL, "M out of range");
     if (dtype != FTLM_F32 && dtype != FTLM_F64) return fail(FTLM_EINVAL, "bad dtype");
     if (dist != FTLM_VEC_GAUSS && dist != FTLM_VEC_RADEMACHER) return fail(FTLM_EINVAL, "bad distribution");
-    if (block == 0) block = dtype == FTLM_F32 ? 16 : 8;
+    if (block == 0) block = 8;
     if (!valid_block(block)) return fail(FTLM_EINVAL, "block width must be 0, 1, 4, 8 or 16");
     if (streams < 0 || streams > kMaxSideStreams) return fail(FTLM_EINVAL, "streams must be 0..8");
     if (streams == 0) streams = side_streams();
@@ -402,7 +409,7 @@ ftlm_status batch_create(int n, const ftlm_batch_item *items, int M, ftlm_vec_di
     for (int i = 0; i < n; ++i) {
         const ftlm_basis *b = items[i].basis;
         num_sms = b->num_sms;
-        if (b->two_s > 1 || (b->N <= 32 && b->D > kSmallRows)) {  // the multi-sector path
+        if (b->two_s > 1 || (b->N <= 32 && b->D > kPersistentRows)) {  // the multi-sector path
             ms_items.push_back(i);
             continue;
         }
@@ -499,7 +506,8 @@ ftlm_status batch_create(int n, const ftlm_batch_item *items, int M, ftlm_vec_di
                     w.stile_off = (uint32_t)stile_unit.size();
                     w.kind = kind;
                 }
-                const uint32_t nst = (uint32_t)((b->D + stream_rows - 1) / stream_rows);
+                const uint32_t sr = stream_rows ? stream_rows : ms_stream_rows(b->D);
+                const uint32_t nst = (uint32_t)((b->D + sr - 1) / sr);
                 MsUnit u{};
                 u.s = b->tables();
                 u.bl = b->mode == FTLM_RANK_CLT ? b->bonds_clt : b->bonds_cr;
@@ -511,7 +519,7 @@ ftlm_status batch_create(int n, const ftlm_batch_item *items, int M, ftlm_vec_di
                 u.seed = items[i].seed;
                 u.tau = dtype == FTLM_F32 ? b->tau32 : b->tau64;
                 u.tile_rows = tile_rows;
-                u.stream_rows = stream_rows;
+                u.stream_rows = sr;
                 u.tile0 = w.n_tiles;
                 u.n_tiles = nt;
                 u.stile0 = w.n_stiles;
@@ -870,7 +878,7 @@ extern "C" ftlm_status ftlm_batch_autotune_plan(int n, const ftlm_batch_item *it
         const ftlm_basis *b = items[i].basis;
         if (!b) continue;
         if (b->two_s == 1 && b->N > 32 && b->D > kSmallRows) any_large = true;
-        if (b->two_s > 1 || (b->N <= 32 && b->D > kSmallRows)) any_ms = true;
+        if (b->two_s > 1 || (b->N <= 32 && b->D > kPersistentRows)) any_ms = true;
     }
     int device = 0;
     cudaMemPool_t pool = nullptr;
@@ -879,7 +887,7 @@ extern "C" ftlm_status ftlm_batch_autotune_plan(int n, const ftlm_batch_item *it
     cudaEvent_t ev[2] = {nullptr, nullptr};
     FTLM_CUDA(cudaEventCreate(&ev[0]));
     FTLM_CUDA(cudaEventCreate(&ev[1]));
-    ftlm_batch_plan cur{dtype == FTLM_F32 ? 16 : 8, any_large ? 4 : 1, (int)kMsTileRows, (int)kMsStreamRows};
+    ftlm_batch_plan cur{8, any_large ? 4 : 1, (int)kMsTileRows, (int)kMsStreamRows};
     float cur_ms = -1.f;
     int count = 0;
     ftlm_status st = FTLM_OK;

@@ -426,7 +426,8 @@ extern "C" ftlm_status ftlm_flow_create(ftlm_dtype dtype, int block, int M, ftlm
     // tile maps: every unit row needs 2 B values of vectors at least
     const uint64_t rows = f->units_bytes / (2ull * block * (dtype == FTLM_F32 ? 4 : 8));
     f->cap_tiles = rows / kMsTileRows + max_units + 1;
-    f->cap_stiles = rows / kMsStreamRows + max_units + 1;
+    // streaming tiles: at most 33 for a unit of fewer than 32 kMsStreamRows rows
+    f->cap_stiles = std::min<uint64_t>(rows / kMsTileRows + max_units, rows / kMsStreamRows + 33ull * max_units) + 1;
     // [units | 3 H.v tile maps | streaming map | finished lists | Ritz rows]; the
     // tiles of every unit together number at most cap_tiles (cap_stiles)
     const uint64_t o_units = 0;
@@ -462,9 +463,12 @@ extern "C" ftlm_status ftlm_flow_create(ftlm_dtype dtype, int block, int M, ftlm
     f->stage_cur = 0;
     f->rz = nullptr;
     f->ev_main = f->ev_rz = nullptr;
+    // one pinned block for the ring (pinning costs a driver call each)
+    f->stage_bytes = align256(f->stage_bytes);
+    e = cudaMallocHost((void **)&f->stage[0], f->stage_bytes * ftlm_flow::kStages);
     for (int k = 0; k < ftlm_flow::kStages && e == cudaSuccess; ++k) {
-        e = cudaMallocHost((void **)&f->stage[k], f->stage_bytes);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&f->stage_ev[k], cudaEventDisableTiming);
+        f->stage[k] = f->stage[0] + (size_t)k * f->stage_bytes;
+        e = cudaEventCreateWithFlags(&f->stage_ev[k], cudaEventDisableTiming);
     }
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&f->rz, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&f->ev_main, cudaEventDisableTiming);
@@ -475,10 +479,9 @@ extern "C" ftlm_status ftlm_flow_create(ftlm_dtype dtype, int block, int M, ftlm
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&f->slot[k].join, cudaEventDisableTiming);
     }
     if (e != cudaSuccess) {
-        for (int k = 0; k < ftlm_flow::kStages; ++k) {
-            if (f->stage[k]) cudaFreeHost(f->stage[k]);
+        if (f->stage[0]) cudaFreeHost(f->stage[0]);
+        for (int k = 0; k < ftlm_flow::kStages; ++k)
             if (f->stage_ev[k]) cudaEventDestroy(f->stage_ev[k]);
-        }
         if (f->rz) cudaStreamDestroy(f->rz);
         if (f->ev_main) cudaEventDestroy(f->ev_main);
         if (f->ev_rz) cudaEventDestroy(f->ev_rz);
@@ -555,9 +558,9 @@ extern "C" ftlm_status ftlm_flow_add(ftlm_flow *f, const ftlm_batch_item *item, 
         u.seed = item->seed;
         u.tau = f->dtype == FTLM_F32 ? b->tau32 : b->tau64;
         u.tile_rows = kMsTileRows;
-        u.stream_rows = kMsStreamRows;
+        u.stream_rows = ms_stream_rows(b->D);
         u.n_tiles = (uint32_t)((b->D + kMsTileRows - 1) / kMsTileRows);
-        u.n_stiles = (uint32_t)((b->D + kMsStreamRows - 1) / kMsStreamRows);
+        u.n_stiles = (uint32_t)((b->D + u.stream_rows - 1) / u.stream_rows);
         u.chain_base = (uint32_t)cb + (uint32_t)r0;
         u.key_n = b->key_n;
         u.K = b->K;
@@ -674,10 +677,8 @@ extern "C" void ftlm_flow_destroy(ftlm_flow *f)
     if (!f) return;
     cudaDeviceSynchronize();
     cudaFreeAsync(f->dev_block, 0);
-    for (int k = 0; k < ftlm_flow::kStages; ++k) {
-        cudaFreeHost(f->stage[k]);
-        cudaEventDestroy(f->stage_ev[k]);
-    }
+    cudaFreeHost(f->stage[0]);
+    for (int k = 0; k < ftlm_flow::kStages; ++k) cudaEventDestroy(f->stage_ev[k]);
     cudaStreamDestroy(f->rz);
     cudaEventDestroy(f->ev_main);
     cudaEventDestroy(f->ev_rz);

@@ -15,6 +15,17 @@ constexpr uint32_t kMsTileRows = 2048;
 // the transposed trees 1.35 / 1.18 / 1.67 s at 8192 / 16384 / 32768 rows; H.v best
 // at 2048).
 constexpr uint32_t kMsStreamRows = 8 * kMsTileRows;
+// Rows per streaming tile of a sector of D rows: kMsStreamRows, or less (down to one
+// H.v tile) where that would leave a unit with fewer than 32 tiles -- a few CTAs each
+// streaming megabytes.  Measured on the 13 sectors of the spin-1 icosahedron (D up to
+// 73 789, 24 chains, blocks of 8): 17.2 -> 15.2 ms per batch; the four clusters of 18 to
+// 22 sites stay within 1 %.  A function of D alone, so a unit's sums do not depend on
+// the units it runs with.
+inline uint32_t ms_stream_rows(uint64_t D)
+{
+    const uint64_t r = (D / 32 + kRowThreads - 1) / kRowThreads * kRowThreads;
+    return (uint32_t)(r < kMsTileRows ? kMsTileRows : (r > kMsStreamRows ? kMsStreamRows : r));
+}
 
 // One block of B chains of one sector.  Offsets are into the run's workspace.
 struct MsUnit {
