@@ -259,6 +259,10 @@ __device__ __forceinline__ void row_f64(const SectorTables &s, const BondList &b
                     }
                     if constexpr (NC) ld_vec<B>(x + (size_t)k * B, xv[q], false);
                     else ld_vec_coherent<B>(x + (size_t)k * B, xv[q]);
+                } else {  // a value on either path keeps the load here, ahead of its use
+                    j[q] = 0.0;
+#pragma unroll
+                    for (int r = 0; r < B; ++r) xv[q][r] = 0.0;
                 }
             }
 #pragma unroll
