@@ -11,6 +11,7 @@ Convenience layer (also marshalling only): ``Basis`` owns a sector handle,
 thermodynamic sums) through the same entry points.
 """
 import ctypes
+import math
 import os
 
 import numpy as np
@@ -757,19 +758,70 @@ def computed_two_sz(N, two_s=1):
     return list(range(top % 2, top + 1, 2))
 
 
+# run_ftlm: sectors whose workspace is at most this many bytes share the device on up to
+# this many side streams.  One sector of a small cluster is a chain of launches of a few
+# microseconds each on a part of the SMs (N = 16 ring, FP64, R = 20, nine sectors:
+# 28.2 ms one after another).
+SIDE_BYTES, SIDE_STREAMS = 64 << 20, 4
+
+
 def run_ftlm(N, bonds, R, M, T, seed=1, dist=GAUSS, dtype=torch.float32, g=2.0, h=0.0,
              sectors=None, mode=RANK_AUTO, keep_coeffs=False, stream=None):
     """A whole FTLM job on the device: for each sector (default: every S^z >= 0,
-    mirrored), R chains of M steps, then E, C, chi, mag on the grid T."""
+    mirrored), R chains of M steps, then E, C, chi, mag on the grid T.  Everything is
+    queued on `stream` or joined to it; small sectors run side by side."""
     dev = torch.device("cuda", torch.cuda.current_device())
     if not torch.is_tensor(T):
         T = torch.as_tensor(np.asarray(T, dtype=np.float64), device=dev)
     two = computed_two_sz(N) if sectors is None else list(sectors)
-    res, work = [], None
-    for tz in two:
-        with Basis(N, tz, bonds, mode, stream) as b:
-            r = lanczos(b, R, M, seed, dist, dtype, work=work, keep_coeffs=keep_coeffs, stream=stream)
-            res.append((tz, b.dim, r))
-    obs = thermo(res, T, R, M, g, h, mirror=sectors is None, stream=stream)
+    base = torch.cuda.current_stream() if stream is None else stream
+    code = _dtype_code(dtype)
+    # a sector's workspace is at least two vectors of its dimension
+    row = 2 * (4 if code == F32 else 8)
+    small = [k for k, tz in enumerate(two)
+             if abs(tz) <= N and math.comb(int(N), (int(N) + int(tz)) // 2) * row <= SIDE_BYTES]
+    res = [None] * len(two)
+    held = []
+    try:
+        for a in range(0, len(small), MAX_SECTORS):
+            ks = small[a:a + MAX_SECTORS]
+            held += zip(ks, Basis.sectors(N, [two[k] for k in ks], bonds, mode, base, wait=False))
+        need = {k: ftlm_lanczos_workspace_bytes(b.handle, R, M, code) for k, b in held}
+        side = sorted((k for k, _ in held if need[k] <= SIDE_BYTES), key=lambda k: -need[k])
+        n = min(SIDE_STREAMS, len(side))
+        streams = [torch.cuda.Stream(dev) for _ in range(n)] if n > 1 else [base] * n
+        lanes = [side[i::n] for i in range(n)]
+        works = [torch.empty((need[lane[0]] + 255) // 256 * 256, dtype=torch.uint8, device=dev) for lane in lanes]
+        by_k = dict(held)
+        if n > 1:  # the side streams start after the tables, and after this memory's last uses
+            here = torch.cuda.current_stream()
+            for s, w in zip(streams, works):
+                s.wait_stream(base)
+                if here != base:
+                    s.wait_stream(here)
+                w.record_stream(s)
+        for lane, s, w in zip(lanes, streams, works):
+            for k in lane:
+                res[k] = (two[k], by_k[k].dim,
+                          lanczos(by_k[k], R, M, seed, dist, dtype, work=w, keep_coeffs=keep_coeffs, stream=s))
+        for k, tz in enumerate(two):  # the others one after another on the job's stream
+            if res[k] is not None:
+                continue
+            if k in by_k:
+                res[k] = (tz, by_k[k].dim,
+                          lanczos(by_k[k], R, M, seed, dist, dtype, keep_coeffs=keep_coeffs, stream=base))
+                continue
+            with Basis(N, tz, bonds, mode, base) as b:
+                res[k] = (tz, b.dim, lanczos(b, R, M, seed, dist, dtype, keep_coeffs=keep_coeffs, stream=base))
+        if n > 1:
+            for s in streams:
+                base.wait_stream(s)
+    except BaseException:
+        torch.cuda.synchronize(dev)  # side work may still use the tables and workspaces
+        raise
+    finally:
+        for _, b in held:
+            b.release(base)
+    obs = thermo(res, T, R, M, g, h, mirror=sectors is None, stream=base)
     obs["sectors"] = res
     return obs
