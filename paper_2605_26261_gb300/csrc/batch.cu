@@ -165,7 +165,7 @@ batch_kernel(const BatchItemDev *__restrict__ items, const BatchUnitDev *__restr
                 V out[B];
 #pragma unroll
                 for (int r = 0; r < B; ++r) {
-                    out[r] = r < (int)un.nact ? (V)start_value(key[r], t, dist) : (V)0;
+                    out[r] = r < (int)un.nact ? start_entry<V>(key[r], t, dist) : (V)0;
                     acc[r].add(out[r], out[r]);
                 }
                 st_vec<B>(u0 + (size_t)t * B, out);

@@ -70,8 +70,7 @@ start_kernel(uint32_t D, const KeySpec keys, int dist, const double *__restrict_
         V out[B];
 #pragma unroll
         for (int r = 0; r < B; ++r) {
-            const double v = src ? src[(size_t)r * D + t] : start_value(s_key[r], t, dist);
-            out[r] = (V)v;
+            out[r] = src ? (V)src[(size_t)r * D + t] : start_entry<V>(s_key[r], t, dist);
             acc[r].add(out[r], out[r]);
         }
         st_vec<B>(u + (size_t)t * B, out);

@@ -96,7 +96,7 @@ ms_start_kernel(const MsUnit *__restrict__ units, const uint32_t *__restrict__ t
             V out[B];
 #pragma unroll
             for (int r = 0; r < B; ++r) {
-                out[r] = r < U.nact ? (V)start_value(key[r], t, dist) : (V)0;
+                out[r] = r < U.nact ? start_entry<V>(key[r], t, dist) : (V)0;
                 acc[r].add(out[r], out[r]);
             }
             st_vec<B>(u0 + (size_t)t * B, out);
