@@ -232,6 +232,46 @@ __device__ __forceinline__ void tiles_done(const EpiDev &ep, AlphaSums<B, THREAD
     }
 }
 
+// The same with alpha_j formed by the last CTA to arrive, from one pair of words per CTA and
+// chain in ep.partials (2 B words per CTA of the grid).
+template <int B, int THREADS>
+__device__ __forceinline__ void tiles_end(const EpiDev &ep, AlphaSums<B, THREADS> &s)
+{
+    constexpr uint32_t W = 2 * B;
+    static_assert(THREADS % W == 0, "a slice of the CTAs per W threads");
+    __shared__ bool s_last;
+    unsigned long long *part = reinterpret_cast<unsigned long long *>(ep.partials);
+    __syncthreads();
+    if (threadIdx.x < W) {
+        long long v = 0;
+#pragma unroll
+        for (int w = 0; w < THREADS / 32; ++w) v += s.v[w][threadIdx.x];
+        part[(size_t)blockIdx.x * W + threadIdx.x] = (unsigned long long)v;
+        if (threadIdx.x == 0 && s.bad) atomicOr(ep.counter + 3, s.bad);
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(ep.counter, 1u) == gridDim.x - 1;
+    if (threadIdx.x < W) s.v[0][threadIdx.x] = 0;
+    __syncthreads();
+    if (!s_last) return;
+    unsigned long long v = 0;
+    for (uint32_t g = threadIdx.x / W; g < gridDim.x; g += THREADS / W) v += __ldcg(part + (size_t)g * W + threadIdx.x % W);
+    atomicAdd(reinterpret_cast<unsigned long long *>(&s.v[0][threadIdx.x % W]), v);
+    __syncthreads();
+    if (threadIdx.x < B) {
+        const int r = threadIdx.x;
+        const bool bad = (__ldcg(ep.counter + 3) >> r) & 1u;
+        const double a = ((double)s.v[0][2 * r] + (double)s.v[0][2 * r + 1] * 0x1p-40) * ep.unscale;
+        if (!ep.st[r].stopped) {
+            ep.st[r].alpha = bad ? NAN : a;
+            ep.alpha_out[(size_t)r * ep.alpha_stride] = bad ? NAN : a;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) ep.counter[0] = ep.counter[1] = ep.counter[3] = 0;
+}
+
 // End of a launch that takes its tiles in dynamic order and leaves no sums (walk A).
 __device__ __forceinline__ void tiles_done(const EpiDev &ep, uint32_t nwarps)
 {

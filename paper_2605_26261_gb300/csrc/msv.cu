@@ -29,7 +29,7 @@ namespace {
 
 // The bonds of a general-spin unit in shared memory.
 struct SpinBonds {
-    uint4 e[kMaxBondSlots];
+    uint4 e[kSpinMaxBonds];
 };
 
 struct UnitView {
@@ -121,12 +121,23 @@ ms_start_kernel(const MsUnit *__restrict__ units, const uint32_t *__restrict__ t
 // Step j: y = H q_j - beta_{j-1} q_{j-1} over the u_{j-1} block and alpha_j, for
 // every tile of every unit (x = u_j is block (j - 1) % 2, y block j % 2).
 // Resident CTAs per SM the registers are cut for: FP32 blocks up to 8 fit 3 CTAs
-// without spills (FP64 blocks of 4 and 8 need 2), single vectors 4 (3 for FP64
-// general-spin rows).
+// without spills (FP64 blocks of 4 and 8 need 2, general-spin blocks of 4 fit 3), single
+// vectors 4 (3 for FP64 general-spin rows).
 template <typename V, int B, int KIND> __host__ __device__ constexpr int ms_min_ctas()
 {
-    return B >= 16 ? 1
-                   : (sizeof(V) == 8 && B >= 4 ? 2 : (B >= 4 ? 3 : (sizeof(V) == 8 && KIND == kMsSpin ? 3 : 4)));
+    if (B >= 16) return 1;
+    if (sizeof(V) == 8 && KIND == kMsSpin) return B >= 8 ? 2 : 3;
+    if (sizeof(V) == 8 && B >= 4) return 2;
+    return B >= 4 ? 3 : 4;
+}
+
+// Dynamic shared memory of the H.v kernel: the low-block rank table, and the lists of its
+// warps (spin_rows.cuh).
+template <typename V> constexpr size_t ms_hv_smem(int kind)
+{
+    return kind == kMsClt ? 0
+                          : kSpinMaxLow * sizeof(uint16_t) +
+                                (kind == kMsSpin ? kRowThreads / 32 * spin_list_bytes<V>(kSpinMaxHH, kSpinMaxCross) : 0);
 }
 
 template <typename V, int KIND, int B, int C>
@@ -135,9 +146,9 @@ ms_hv_kernel(const MsUnit *__restrict__ units, const uint32_t *__restrict__ tile
              int M, double *alpha, char *ws)
 {
     constexpr bool CLT = KIND == kMsClt, SPIN = KIND == kMsSpin;
-    extern __shared__ uint16_t s_tlo[];
+    extern __shared__ __align__(16) uint16_t s_tlo[];
     __shared__ typename std::conditional<SPIN, SpinBonds, RowBonds<V, uint32_t>>::type s_bond;
-    __shared__ V s_J[SPIN ? kMaxBondSlots : 1];
+    __shared__ V s_J[SPIN ? kSpinMaxBonds : 1];
     __shared__ V s_cf[SPIN ? kSpinCoef : 1];
     __shared__ V s_inv_s[B], s_c_prev[B];
     __shared__ int s_skip;
@@ -195,7 +206,8 @@ ms_hv_kernel(const MsUnit *__restrict__ units, const uint32_t *__restrict__ tile
             const uint32_t t = ok ? tt : D - 1;  // rows past the end recompute the last row, unstored
             if constexpr (SPIN) {
                 V acc[B], diag;
-                spin_row<V, B, C, false>(U.s, U.spin, s_tlo, nullptr, s_bond.e, s_J, s_cf, x, t, acc, diag);
+                spin_row<V, B, C>(U.s, U.spin, s_tlo, s_bond.e, s_J, s_cf,
+                                  spin_list<V>(U.spin, s_tlo + kSpinMaxLow), true, x, t, acc, diag);
                 if (ok) epi_row<V, B, true>(ep, s_inv_s, s_c_prev, x, y, t, diag, acc, apart);
             } else {
                 V acc[B], dsum;
@@ -346,7 +358,7 @@ template <int B> __host__ __device__ constexpr int ms_chunk() { return B >= 8 ? 
 
 template <typename V, int B> void *ms_hv_ptr(int kind)
 {
-    if (kind == kMsSpin) return (void *)ms_hv_kernel<V, kMsSpin, B, spin_chunk<B>()>;
+    if (kind == kMsSpin) return (void *)ms_hv_kernel<V, kMsSpin, B, 1>;
     if (kind == kMsClt) return (void *)ms_hv_kernel<V, kMsClt, B, ms_chunk<B>()>;
     return (void *)ms_hv_kernel<V, kMsCr, B, ms_chunk<B>()>;
 }
@@ -356,7 +368,7 @@ ftlm_status ms_run_typed(const MsWave &w, const MsUnit *units, const uint32_t *t
                          const uint32_t *stile_unit, int M, int dist, char *ws, double *alpha, double *beta,
                          int *meff, int num_sms, cudaStream_t stream)
 {
-    const size_t smem = w.kind == kMsClt ? 0 : ((size_t)1 << kLoBitsMax) * sizeof(uint16_t);
+    const size_t smem = ms_hv_smem<V>(w.kind);
     void *hv = ms_hv_ptr<V, B>(w.kind);
     int oh = 1, occ_start = 1, occ_upd = 1;
     FTLM_CUDA(kernel_occupancy(hv, kRowThreads, smem, smem != 0, &oh));
@@ -430,7 +442,7 @@ template <typename V, int B>
 ftlm_status flow_hv_typed(int kind, const MsUnit *units, const uint32_t *tile_unit, uint32_t n_tiles, int j, int M,
                           double *alpha, char *ws, int num_sms, cudaStream_t stream)
 {
-    const size_t smem = kind == kMsClt ? 0 : ((size_t)1 << kLoBitsMax) * sizeof(uint16_t);
+    const size_t smem = ms_hv_smem<V>(kind);
     void *hv = ms_hv_ptr<V, B>(kind);
     int oh = 1;
     FTLM_CUDA(kernel_occupancy(hv, kRowThreads, smem, smem != 0, &oh));

@@ -63,60 +63,87 @@ struct Dims {
     uint64_t at(int m, int a) const { return (a < 0 || a > amax) ? 0 : v[(size_t)m * (amax + 1) + a]; }
 };
 
-// Resident CTAs per SM the registers are capped for; build option
-// FTLM_SPIN_B8_MIN_CTAS for B >= 8 (FP64 blocks of 4: 2, other blocks: 3).
-#ifndef FTLM_SPIN_B8_MIN_CTAS
-#define FTLM_SPIN_B8_MIN_CTAS 2
-#endif
-
-// High-block rank tables up to this many entries (64 KB) are staged in shared
-// memory next to tlo, taking the lookup of the high half of a source rank off the
-// global load path; build option FTLM_SPIN_SMEM_HIGH (0: never).
-#ifndef FTLM_SPIN_SMEM_HIGH
-#define FTLM_SPIN_SMEM_HIGH 16384
-#endif
-constexpr uint64_t kSpinSmemHigh = FTLM_SPIN_SMEM_HIGH;
-
-template <typename V, bool LANCZOS, int B, bool TS>
-__global__ void __launch_bounds__(kRowThreads, B >= 8 ? FTLM_SPIN_B8_MIN_CTAS : (sizeof(V) == 8 && B >= 4 ? 2 : 3))
-hv_spin_kernel(const SectorTables s, const SpinDev p, const V *__restrict__ x0, V *y0, const EpiDev ep0)
+// Launch shapes.  The gathers of a sector of many rows wait on L2 and HBM, and what counts
+// is how many of them an SM has in flight: one bond at a time with 64 registers, so
+// 32 warps per SM.  A sector of few rows (FEW: a few tiles per warp) is bound by the
+// latency of a tile instead and takes more bonds at a time: 2 with 24 warps per SM for
+// blocks of 8, 4 for narrower ones.  FP32 only: rows of doubles are bound by the FP64 pipe
+// and best with 32 warps throughout (blocks of 4, spin-3/2, N = 10: 125 -> 80 us).
+// us per Lanczos H.v launch, S^z = 0 or 1/2, many / few shape:
+//   blocks of 8: s=1 N=13 43.1 / 37.9, N=14 73.9 / 72.4, s=2 N=10 86.9 / 87.9, s=1 N=16 521 / 542
+//   blocks of 4: s=1 N=13 36.9 / 32.7, N=14 59.9 / 59.2, s=2 N=11 273 / 284, s=1 N=16 390 / 416
+//   vectors:     s=1 N=14 54.9 / 48.8, s=2 N=10 66.3 / 60.2, N=11 210 / 212, s=1 N=16 305 / 318
+// Three bonds at a time in 16 warps per SM, with thi in shared memory and no lists, took
+// 39.3, 80.4, 91.9, 656; 34.2, 68.2, 320, 515; 56.5, 66.6, 238, 389 us.
+template <typename V, int B, bool FEW> __host__ __device__ constexpr int spin_min_ctas()
 {
-    constexpr int C = spin_chunk<B>();
+    return B >= 16 || (sizeof(V) == 8 && B >= 8) ? 2 : (FEW ? 3 : 4);
+}
+template <int B, bool FEW> __host__ __device__ constexpr int spin_chunk()
+{
+    return FEW ? (B >= 8 ? 2 : 4) : 1;
+}
+constexpr uint64_t kFewTilesBlock = 128, kFewTilesVector = 512, kListTiles = 64;  // tiles of 32 rows per SM
+
+// MODE: y = H x; the fused Lanczos step with a fixed order of rows; or with tiles handed out
+// by a counter, so that the warps work on one frontier of rows and their gathers share
+// L2: spin-2 icosahedron (628 MB of vectors), blocks of 8 floats, 2946 us in fixed order,
+// 1953 with the counter.  Doubles keep the fixed order: the FP64 work of the sums per
+// tile costs more (14.0 -> 14.3 ms, blocks of 4); so do FP32 vectors and blocks of 4 of
+// few rows, where the counter itself is the bottleneck (s=1, N=13: 27 -> 36 us).
+enum { kSpinPlain = 0, kSpinFixed = 1, kSpinTiles = 2 };
+
+template <typename V, int MODE, int B, bool FEW>
+__global__ void __launch_bounds__(kRowThreads, spin_min_ctas<V, B, FEW>())
+hv_spin_kernel(const SectorTables s, const SpinDev p, const V *__restrict__ x, V *y, const EpiDev ep0, const bool lists)
+{
+    constexpr bool LANCZOS = MODE != kSpinPlain, TILES = MODE == kSpinTiles;
     const EpiDev ep = LANCZOS ? epi_block<B>(ep0) : ep0;
-    const V *__restrict__ x = LANCZOS ? block_ptr(x0, ep0.slot) : x0;
-    V *y = LANCZOS ? block_ptr(y0, ep0.slot) : y0;
-    extern __shared__ uint16_t s_tlo[];
-    // thi after tlo, at a 16-byte boundary (tlo has at most 2^14 entries)
-    uint32_t *s_thi = reinterpret_cast<uint32_t *>(s_tlo + (((size_t)s.lomask + 8) & ~(size_t)7));
-    __shared__ uint4 s_bond[kMaxBondSlots];
-    __shared__ V s_J[kMaxBondSlots];
+    if (LANCZOS) {
+        x = block_ptr(x, ep0.slot);
+        y = block_ptr(y, ep0.slot);
+    }
+    extern __shared__ __align__(16) uint16_t s_tlo[];
+    __shared__ uint4 s_bond[kSpinMaxBonds];
+    __shared__ V s_J[kSpinMaxBonds];
     __shared__ V s_cf[kSpinCoef];
     __shared__ V s_inv_s[B], s_c_prev[B];
+    __shared__ AlphaSums<TILES ? B : 1, kRowThreads> s_asum;
     if (LANCZOS && epi_begin<V, B>(ep, s_inv_s, s_c_prev)) return;
+    if constexpr (TILES) tiles_begin(s_asum);
     for (uint32_t i = threadIdx.x; i < p.nb; i += blockDim.x) {
         s_bond[i] = p.slots[i];
         s_J[i] = spin_J<V>(p)[i];
     }
     spin_stage_coef<V>(p, s_cf);
     for (uint32_t i = threadIdx.x; i <= s.lomask; i += blockDim.x) s_tlo[i] = __ldg(s.tlo + i);
-    if (TS)
-        for (uint32_t i = threadIdx.x; i < s.H; i += blockDim.x) s_thi[i] = __ldg(s.thi + i);
     __syncthreads();
 
+    const SpinList<V> list = spin_list<V>(p, s_tlo + spin_tlo_entries(s));
     DotAcc<V> apart[B];
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
     const uint32_t ntiles = (uint32_t)(((uint64_t)s.D + 31u) / 32u);
-    for (uint32_t tile = warp; tile < ntiles; tile += nwarps) {
+    for (uint32_t tile = warp; tile < ntiles;) {
+        const uint32_t claim = TILES ? claim_tile(ep) : 0u;
         const uint32_t tt = tile * 32u + lane;
         const bool ok_row = tt < s.D;
         const uint32_t t = ok_row ? tt : s.D - 1;  // rows past the end recompute the last row, unstored
         V acc[B], diag;
-        spin_row<V, B, C, TS>(s, p, s_tlo, s_thi, s_bond, s_J, s_cf, x, t, acc, diag);
-        if (ok_row) epi_row<V, B, LANCZOS>(ep, s_inv_s, s_c_prev, x, y, t, diag, acc, apart);
+        spin_row<V, B, spin_chunk<B, FEW>()>(s, p, s_tlo, s_bond, s_J, s_cf, list, lists, x, t, acc, diag);
+        if constexpr (TILES) {
+            DotAcc<V> tacc[B];
+            if (ok_row) epi_row<V, B, true>(ep, s_inv_s, s_c_prev, x, y, t, diag, acc, tacc);
+            add_tile<V, B>(ep, s_asum, tacc);
+            tile = claimed_tile(claim, nwarps);
+        } else {
+            if (ok_row) epi_row<V, B, LANCZOS>(ep, s_inv_s, s_c_prev, x, y, t, diag, acc, apart);
+            tile += nwarps;
+        }
     }
-    if (LANCZOS) epi_end<V, B, kRowThreads>(ep, apart);
+    if constexpr (TILES) tiles_end(ep, s_asum);
+    else if constexpr (LANCZOS) epi_end<V, B, kRowThreads>(ep, apart);
 }
 
 __global__ void spin_labels_kernel(SectorTables s, SpinDev p, uint64_t low_size, uint64_t first, uint64_t count,
@@ -125,7 +152,7 @@ __global__ void spin_labels_kernel(SectorTables s, SpinDev p, uint64_t low_size,
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < count;
          i += (uint64_t)gridDim.x * blockDim.x) {
         SpinRow w;
-        spin_unrank<false>(s, p, nullptr, (uint32_t)(first + i), w);
+        spin_unrank(s, p, (uint32_t)(first + i), w);
         out[i] = (uint64_t)w.hi * low_size + w.lo;
     }
 }
@@ -159,36 +186,58 @@ int grid_of(const ftlm_basis *b, uint64_t n)
     return (int)std::max<uint64_t>(1, std::min(g, cap));
 }
 
-template <typename V, bool LANCZOS, int B>
-ftlm_status launch_spin(const ftlm_basis *b, const V *x, V *y, const EpiDev &ep, int blocks, cudaStream_t stream)
+template <typename V, int MODE, int B, bool FEW>
+ftlm_status launch_spin_mode(const ftlm_basis *b, const V *x, V *y, const EpiDev &ep, int blocks, cudaStream_t stream)
 {
-    const bool ts = b->H <= kSpinSmemHigh;
-    auto kern = ts ? hv_spin_kernel<V, LANCZOS, B, true> : hv_spin_kernel<V, LANCZOS, B, false>;
-    const size_t tlo_bytes = (((size_t)b->tables().lomask + 8) & ~(size_t)7) * sizeof(uint16_t);
-    const size_t smem_max = kSpinMaxLow * sizeof(uint16_t) + (ts ? kSpinSmemHigh * sizeof(uint32_t) : 0);
+    auto kern = hv_spin_kernel<V, MODE, B, FEW>;
+    constexpr uint32_t kWarps = kRowThreads / 32;
+    const size_t smem_max =
+        kSpinMaxLow * sizeof(uint16_t) + kWarps * spin_list_bytes<V>(kSpinMaxHH, kSpinMaxCross);
     int occ = 1;
     FTLM_CUDA(kernel_occupancy((const void *)kern, kRowThreads, smem_max, true, &occ));
-    const size_t smem = tlo_bytes + (ts ? (size_t)b->H * sizeof(uint32_t) : 0);
-    const int grid = row_grid(b, b->D, occ);
+    const SpinDev &p = b->spin;
+    const size_t smem = spin_tlo_entries(b->tables()) * sizeof(uint16_t) +
+                        kWarps * spin_list_bytes<V>(p.n_hh, p.nb - p.n_ll - p.n_hh);
+    // the sums of dynamically ordered tiles take two words per CTA and chain
+    const int grid = std::min(row_grid(b, b->D, occ), MODE == kSpinTiles ? max_row_grid(b) / 2 : max_row_grid(b));
+    // Listing a tile's high-high and cross bonds lengthens its chain of loads, which little
+    // hides in a sector of about two tiles per warp or less: blocks of 4, s=2 N=9 (39 tiles
+    // per SM) 35.2 us listed, 33.5 not; s=1 N=14 (127 tiles per SM) 59.5 and 59.8, s=1
+    // N=16 391 and 435.
+    const bool lists = b->D >= 32 * kListTiles * b->num_sms;
     void *tok = profile_begin(kProfHv, stream, B * blocks);
-    kern<<<dim3(grid, blocks), kRowThreads, smem, stream>>>(b->tables(), b->spin, x, y, ep);
+    kern<<<dim3(grid, blocks), kRowThreads, smem, stream>>>(b->tables(), p, x, y, ep, lists);
     note_launch();
     profile_end(tok, stream);
     FTLM_CUDA(cudaGetLastError());
     return FTLM_OK;
 }
 
-template <typename V, bool LANCZOS>
-ftlm_status launch_spin_b(const ftlm_basis *b, int B, const void *x, void *y, const EpiDev &ep, int blocks,
-                          cudaStream_t stream)
+template <typename V, int B>
+ftlm_status launch_spin(const ftlm_basis *b, const void *x, void *y, const LanczosHv *epi, cudaStream_t stream)
 {
+    const EpiDev ep = epi_of(epi);
     const V *xv = (const V *)x;
     V *yv = (V *)y;
+    const int n = epi ? epi->blocks : 1;
+    if constexpr (sizeof(V) == 4 && B <= 8) {
+        if (b->D < 32 * (B > 1 ? kFewTilesBlock : kFewTilesVector) * b->num_sms)
+            return epi ? launch_spin_mode<V, B == 8 ? kSpinTiles : kSpinFixed, B, true>(b, xv, yv, ep, n, stream)
+                       : launch_spin_mode<V, kSpinPlain, B, true>(b, xv, yv, ep, n, stream);
+    }
+    return epi ? launch_spin_mode<V, sizeof(V) == 4 ? kSpinTiles : kSpinFixed, B, false>(b, xv, yv, ep, n, stream)
+               : launch_spin_mode<V, kSpinPlain, B, false>(b, xv, yv, ep, n, stream);
+}
+
+template <typename V>
+ftlm_status launch_spin_b(const ftlm_basis *b, int B, const void *x, void *y, const LanczosHv *epi,
+                          cudaStream_t stream)
+{
     switch (B) {
-    case 4: return launch_spin<V, LANCZOS, 4>(b, xv, yv, ep, blocks, stream);
-    case 8: return launch_spin<V, LANCZOS, 8>(b, xv, yv, ep, blocks, stream);
-    case 16: return launch_spin<V, LANCZOS, 16>(b, xv, yv, ep, blocks, stream);
-    default: return launch_spin<V, LANCZOS, 1>(b, xv, yv, ep, blocks, stream);
+    case 4: return launch_spin<V, 4>(b, x, y, epi, stream);
+    case 8: return launch_spin<V, 8>(b, x, y, epi, stream);
+    case 16: return launch_spin<V, 16>(b, x, y, epi, stream);
+    default: return launch_spin<V, 1>(b, x, y, epi, stream);
     }
 }
 
@@ -197,13 +246,8 @@ ftlm_status launch_spin_b(const ftlm_basis *b, int B, const void *x, void *y, co
 ftlm_status launch_hv_spin(const ftlm_basis *b, ftlm_dtype dtype, int B, const void *x, void *y,
                            const LanczosHv *epi, cudaStream_t stream)
 {
-    const EpiDev ep = epi_of(epi);
-    const int n = epi ? epi->blocks : 1;
-    if (dtype == FTLM_F32)
-        return epi ? launch_spin_b<float, true>(b, B, x, y, ep, n, stream)
-                   : launch_spin_b<float, false>(b, B, x, y, ep, n, stream);
-    return epi ? launch_spin_b<double, true>(b, B, x, y, ep, n, stream)
-               : launch_spin_b<double, false>(b, B, x, y, ep, n, stream);
+    return dtype == FTLM_F32 ? launch_spin_b<float>(b, B, x, y, epi, stream)
+                             : launch_spin_b<double>(b, B, x, y, epi, stream);
 }
 
 ftlm_status launch_spin_labels(const ftlm_basis *b, uint64_t first, uint64_t count, uint64_t *out,
