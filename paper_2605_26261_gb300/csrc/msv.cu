@@ -120,15 +120,17 @@ ms_start_kernel(const MsUnit *__restrict__ units, const uint32_t *__restrict__ t
 
 // Step j: y = H q_j - beta_{j-1} q_{j-1} over the u_{j-1} block and alpha_j, for
 // every tile of every unit (x = u_j is block (j - 1) % 2, y block j % 2).
-// Resident CTAs per SM the registers are cut for: FP32 blocks up to 8 fit 3 CTAs
-// without spills (FP64 blocks of 4 and 8 need 2, general-spin blocks of 4 fit 3), single
-// vectors 4 (3 for FP64 general-spin rows).
+// Resident CTAs per SM the registers are cut for: FP32 blocks of 8 fit 3 CTAs
+// without spills (FP64 blocks of 4 and 8 need 2, general-spin blocks of 4 fit 3), narrower
+// ones 4 (FP64 general-spin vectors: 3).  Blocks of 4 floats with 4 against 3: random
+// clusters of 18 to 22 sites 117.7 -> 109.8 ms (lookup table), 3.56 -> 3.29 (combinatorial
+// rank); blocks of 8 with 4: 95.5 -> 94 and 14.1 -> 14.5 ms (24 sites).
 template <typename V, int B, int KIND> __host__ __device__ constexpr int ms_min_ctas()
 {
     if (B >= 16) return 1;
     if (sizeof(V) == 8 && KIND == kMsSpin) return B >= 8 ? 2 : 3;
     if (sizeof(V) == 8 && B >= 4) return 2;
-    return B >= 4 ? 3 : 4;
+    return B >= 8 || (KIND == kMsSpin && B == 4) ? 3 : 4;
 }
 
 // Dynamic shared memory of the H.v kernel: the low-block rank table, and the lists of its

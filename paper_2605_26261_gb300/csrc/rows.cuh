@@ -23,6 +23,7 @@ template <> __device__ __forceinline__ double slot_jh<double>(const uint4 &e)
 // Bond data of one chunk, read once and applied to every row of the thread.
 template <typename V, int C>
 struct Chunk {
+    static_assert(kBondChunk % C == 0, "bond ranges are padded to whole chunks of kBondChunk");
     uint32_t mlo[C], mhi[C];
     V jh[C];
 };
