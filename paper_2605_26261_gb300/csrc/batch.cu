@@ -497,8 +497,11 @@ ftlm_status batch_create(int n, const ftlm_batch_item *items, int M, ftlm_vec_di
             for (int r0 = 0; r0 < items[i].R; r0 += B) {
                 const uint64_t vb = align256(b->D * (uint64_t)B * vsize);
                 const uint32_t nt = (uint32_t)((b->D + tile_rows - 1) / tile_rows);
+                const uint32_t sr = stream_rows ? stream_rows : ms_stream_rows(b->D);
+                const uint32_t nst = (uint32_t)((b->D + sr - 1) / sr);
+                // the partial sums hold the H.v tiles and the streaming tiles in turn
                 const uint64_t ub = 2 * vb + align256(kMaxBlock * sizeof(ChainState) + 64) +
-                                    align256((uint64_t)nt * B * sizeof(double));
+                                    align256((uint64_t)std::max(nt, nst) * B * sizeof(double));
                 if (w.n_units && wbytes + ub > ms_wave_bytes()) close_wave();
                 if (!w.n_units) {
                     w.unit0 = (uint32_t)ms_units.size();
@@ -506,8 +509,6 @@ ftlm_status batch_create(int n, const ftlm_batch_item *items, int M, ftlm_vec_di
                     w.stile_off = (uint32_t)stile_unit.size();
                     w.kind = kind;
                 }
-                const uint32_t sr = stream_rows ? stream_rows : ms_stream_rows(b->D);
-                const uint32_t nst = (uint32_t)((b->D + sr - 1) / sr);
                 MsUnit u{};
                 u.s = b->tables();
                 u.bl = b->mode == FTLM_RANK_CLT ? b->bonds_clt : b->bonds_cr;
