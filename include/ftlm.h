@@ -338,7 +338,7 @@ ftlm_status ftlm_lanczos_noalloc(const ftlm_basis *basis, int R, int M, uint64_t
  *   launch (two launches per Lanczos step: H.v with alpha, update with beta;
  *   per-unit reductions over tiles of 2048 rows for H.v, handed out in order from
  *   a counter, and D / 32 rows, 2048 to 16384, for the update; waves of at most
- *   FTLM_MS_WAVE_MB = 256 MB of vectors) on a stream forked from the caller's.
+ *   FTLM_MS_WAVE_MB = 512 MB of vectors) on a stream forked from the caller's.
  *   Larger spin-1/2 sectors with N > 32 run the launch sequence of ftlm_lanczos with
  *   blocks of up to `block` chains, spread over up to `streams` side streams (1..8;
  *   0 = FTLM_BATCH_STREAMS or 4).  Uploads the plan's descriptors on
@@ -441,9 +441,9 @@ ftlm_status ftlm_batch_autotune(int n_items, const ftlm_batch_item *items, int M
  *   max_units limit right now (nothing is queued: add it again later).
  * ftlm_flow_step -- queue up to `steps` Lanczos steps of every admitted unit on
  *   `stream` (start vectors for the newly admitted ones first).  The units are
- *   visited in waves of consecutive units (admission order) of at most 256 MB of
+ *   visited in waves of consecutive units (admission order) of at most 512 MB of
  *   vectors, each wave running its steps before the next one on its stream starts
- *   (so that a wave's vectors stay in L2 between its steps).  The waves are spread
+ *   (so that more of a wave's vectors stay in L2 between its steps).  The waves are spread
  *   over the flow's wave streams (least loaded first), which start after the work
  *   queued on `stream` and which `stream` waits for at the end of the call: the
  *   launches of different waves overlap (one wave's gathers with another's row

@@ -37,16 +37,19 @@
 
 namespace ftlm {
 
-// Vector bytes of one wave of the multi-sector path: FTLM_MS_WAVE_MB or 256 MB.
-// Small waves keep a wave's vectors near the L2 size (measured on GB300 with 256
-// clusters of 18-22 sites: 256 MB waves 9.6 s per run, 2 GB 11.0 s, 8 GB 11.9 s);
-// a unit larger than the budget forms a wave of its own.
+// Vector bytes of one wave of the multi-sector path: FTLM_MS_WAVE_MB or 512 MB.  A wave's
+// launches end in a tail of tiles, and the waves of a batch come one after another, so
+// few large waves are better, even though 256 MB would stay nearer the L2 size.
+// Blocks of 8 floats, R = 16, M = 100, waves of 128 / 256 / 512 / 1024 MB: 4 clusters
+// of 18 to 22 sites 117 / 95.5 / 87.0 / 86.9 ms; 64 clusters of the many-cluster
+// benchmark - / 1384 / 1303 / 1250 ms; six served jobs 122.7 / 122.4 / 119 / 131 ms (their waves also run on
+// several streams).  A unit larger than the budget forms a wave of its own.
 uint64_t ms_wave_bytes()
 {
     static const uint64_t v = [] {
         const char *e = std::getenv("FTLM_MS_WAVE_MB");
-        const long long mb = e ? std::atoll(e) : 256;
-        return (uint64_t)(mb > 0 ? mb : 256) << 20;
+        const long long mb = e ? std::atoll(e) : 512;
+        return (uint64_t)(mb > 0 ? mb : 512) << 20;
     }();
     return v;
 }

@@ -69,7 +69,7 @@ ftlm_status ms_run_wave(const MsWave &w, ftlm_dtype dtype, int B, const MsUnit *
                         const uint32_t *stile_unit, int M, int dist, char *ws, double *alpha, double *beta,
                         int *meff, int num_sms, cudaStream_t stream);
 
-// Vector bytes per wave of the multi-sector path (FTLM_MS_WAVE_MB, default 256 MB;
+// Vector bytes per wave of the multi-sector path (FTLM_MS_WAVE_MB, default 512 MB;
 // batch.cu), used by batches and by the continuous flow.
 uint64_t ms_wave_bytes();
 

@@ -5,7 +5,7 @@ every S^z >= 0 sector (mirrored), R chains of M Lanczos steps each, then E, C, c
 and <S^z> on a temperature grid (Eq. 6-9; the field enters as -h S^z per sector).
 Jobs arrive at any time.  The chains of every large sector on the device advance
 together through one continuous flow (ftlm_flow_*): the flow visits its sectors in
-waves of at most 256 MB of vectors (L2-sized) and runs a few Lanczos steps of each
+waves of at most 512 MB of vectors and runs a few Lanczos steps of each
 wave with one multi-sector H.v launch per rank kind and one update launch per step,
 whatever step each sector is at.  Between passes the loop admits the sectors of
 waiting jobs, in arrival order, as long as their device memory fits in the flow's
