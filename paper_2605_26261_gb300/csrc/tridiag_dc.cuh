@@ -8,7 +8,7 @@
 // Components with a negligible z and pairs of close d are deflated (Dongarra &
 // Sorensen 1987); the roots of 1/rho + sum_j z_j^2 / (d_j - x) are found one per
 // thread by rational interpolation of the two half sums (Bunch, Nielsen & Sorensen
-// 1978) inside a shrinking bracket, as offsets from the nearer pole, and the
+// 1978; Li 1994) inside a shrinking bracket, as offsets from the nearer pole, and the
 // eigenvectors are those of the z recomputed from the roots, which makes them
 // orthogonal to working accuracy (Gu & Eisenstat 1995).  Only the first and last row
 // of the eigenvector matrix are carried: the last one feeds the z of the next merge,
@@ -21,10 +21,11 @@
 // instructions per pole and root; the merges of all levels cost twice the last one.
 // Measured on GB300, rows of Lanczos coefficients, against implicit QR with one thread
 // per problem (a chain of about m^2 dependent rotations), n problems of m rows: m = 100,
-// n = 8 / 690 / 4096: 21.2 / 21.3 / 21.3 ms -> 0.96 / 2.1 / 11.2 ms; m = 20, n = 8: 0.97
-// -> 0.14 ms; m = 300, n = 8: 180 -> 8.1 ms; only for tens of thousands of problems at
-// once is QR as fast (n = 45072, m = 100: 87 against 116 ms, of a 7 s step).  Without
-// the float estimate (doubles from the middle of the gap) 1.6 ms at m = 100, n = 8.
+// n = 8 / 690 / 4096: 21.2 / 21.3 / 21.3 ms -> 0.53 / 1.5 / 8.4 ms; m = 20, n = 8: 0.97
+// -> 0.15 ms; m = 300, n = 8: 180 -> 4.8 ms; only for tens of thousands of problems at
+// once is QR as fast.  Without the float estimate (doubles from the middle of the gap)
+// 1.6 ms at m = 100, n = 8; with the half-sum steps alone 0.96 ms, 10 to 18 double steps for
+// one or two roots of the last merge.
 //
 // Every step is a phase executed by all threads between two barriers, written as a
 // function of (thread, thread count), so that the same code runs on the host, one
@@ -326,19 +327,43 @@ __host__ __device__ __forceinline__ Halves<float> secular(const Work &w, int lo,
                             [=](int j) { return recip(((dh[j] - oh) + (dl[j] - ol)) - tau); });
 }
 
-// Step from x of the rational model c + S/(d_a - x) + R/(d_b - x) that matches both
-// half sums and their derivatives (da = d_a - x, db = d_b - x, w = f(x)): the root
-// eta of c eta^2 - A eta + da db w = 0 between the two poles (last: to the right of
-// both).
+// Step from x of the rational model c + S/(d_a - x) + R/(d_b - x) with the value w = f(x)
+// (da = d_a - x, db = d_b - x): the root eta of c eta^2 - A eta + da db w = 0 between
+// the two poles (last: to the right of both).
 template <typename F>
-__host__ __device__ __forceinline__ F rational_step(const Halves<F> &h, F irho, F da, F db, F w, bool last)
+__host__ __device__ __forceinline__ F model_root(F c, F S, F R, F da, F db, F w, bool last)
 {
-    const F c = irho + (h.psi - da * h.dpsi) + (h.phi - db * h.dphi);
-    const F A = fma(c, da + db, fma(da * da, h.dpsi, db * db * h.dphi));
+    const F A = fma(c, da + db, S + R);
     const F B = da * db * w;
     const F disc = sqrt(fmax((F)0, fma(A, A, (F)-4 * c * B)));
     const F sd = last ? -disc : disc;
-    return (last ? A >= (F)0 : A <= (F)0) ? (A - sd) / ((F)2 * c) : (F)2 * B / (A + sd);
+    const bool minus = last ? A >= (F)0 : A <= (F)0;  // the quotient without cancellation
+    return (minus ? A - sd : (F)2 * B) * recip(minus ? (F)2 * c : A + sd);
+}
+// The weights that match both half sums and their derivatives (Bunch, Nielsen & Sorensen).
+template <typename F>
+__host__ __device__ __forceinline__ F rational_step(const Halves<F> &h, F da, F db, F w, bool last)
+{
+    return model_root<F>(w - da * h.dpsi - db * h.dphi, da * da * h.dpsi, db * db * h.dphi, da, db, w, last);
+}
+// The near pole's own weight z^2 (near_z: z of pole a if near_a, else of b), the other one
+// matching the rest of the derivative (Li 1994).  The step above attributes far poles' part
+// of the derivative to a near pole of tiny z and then only halves the distance; this one
+// is exact there.  Ghosts of Lanczos coefficients have such roots in the last merges.
+template <typename F>
+__host__ __device__ __forceinline__ F fixed_step(const Halves<F> &h, F da, F db, F w, bool last, bool near_a, F near_z)
+{
+    const F dn = near_a ? da : db, df = near_a ? db : da;
+    const F q = near_z * recip(dn), rest = fmax((F)0, h.dpsi + h.dphi - q * q);
+    const F zz = near_z * near_z, rr = df * df * rest;
+    return model_root<F>(w - near_z * q - df * rest, near_a ? zz : rr, near_a ? rr : zz, da, db, w, last);
+}
+
+// A point inside a bracket: one that reaches the pole is cut by a factor, not by its
+// middle.
+template <typename F> __host__ __device__ __forceinline__ F cut(F lb, F ub)
+{
+    return lb == (F)0 ? (F)0.0625 * ub : (ub == (F)0 ? (F)0.0625 * lb : (F)0.5 * (lb + ub));
 }
 
 // A float estimate of the root between poles a and b (last: above b) and the pole to
@@ -348,10 +373,11 @@ __host__ __device__ inline float root_estimate(const Work &w, int lo, int hi, in
                                                float rho, int &o)
 {
     const float irho = 1.f / rho;
-    float x;
+    float x, lb = 0.f, ub = 0.f;  // bracket, as offsets from pole o
     if (last) {
         o = b;
         x = 0.5f * rho;
+        ub = rho * 1.01f;
     } else {
         const float half = 0.5f * ((w.dh[b] - w.dh[a]) + (w.dl[b] - w.dl[a]));
         const Halves<float> h = secular(w, lo, a, hi, c, a, half);
@@ -359,24 +385,32 @@ __host__ __device__ inline float root_estimate(const Work &w, int lo, int hi, in
         // f rises from -inf at d[a] to +inf at d[b]: the sign at the middle tells the
         // nearer pole
         o = v >= 0.f ? a : b;
-        x = (v >= 0.f ? half : -half) + rational_step(h, irho, -half, half, v, false);
+        lb = v >= 0.f ? 0.f : -half;
+        ub = v >= 0.f ? half : 0.f;
+        x = (v >= 0.f ? half : -half) + rational_step(h, -half, half, v, false);
     }
-    for (int it = 0; it < 6; ++it) {
+    const float x0 = 0.5f * (lb + ub);
+    for (int it = 0; it < 16; ++it) {
         const float da = ((w.dh[a] - w.dh[o]) + (w.dl[a] - w.dl[o])) - x;
         const float db = ((w.dh[b] - w.dh[o]) + (w.dl[b] - w.dl[o])) - x;
         const Halves<float> h = secular(w, lo, a, hi, c, o, x);
-        const float eta = rational_step(h, irho, da, db, irho + h.psi + h.phi, last);
-        x += eta;
-        if (!(fabs(eta) > 1e-4f * fabs(x))) break;
+        const float v = irho + h.psi + h.phi;
+        if (it < 4) {
+            const float eta = rational_step(h, da, db, v, last);
+            x += eta;
+            if (!(fabs(eta) > 1e-4f * fabs(x))) break;
+            if (it == 3 && !(x > lb && x < ub)) x = x0;
+        } else {  // one of the slow roots: inside the bracket from here on
+            if (v < 0.f) lb = x;
+            else ub = x;
+            float y = x + fixed_step(h, da, db, v, last, o == a, w.zh[o]);
+            if (!(y > lb && y < ub)) y = cut(lb, ub);
+            const bool done = fabs(y - x) <= 1e-4f * fabs(y);
+            x = y;
+            if (done) break;
+        }
     }
     return x;
-}
-
-// A point inside a bracket: one that reaches the pole is cut by a factor, not by its
-// middle.
-__host__ __device__ __forceinline__ double cut(double lb, double ub)
-{
-    return lb == 0.0 ? 0.0625 * ub : (ub == 0.0 ? 0.0625 * lb : 0.5 * (lb + ub));
 }
 
 // Root `i` of the block with poles lo .. hi-1: its pole `o` and offset tau.  Returns
@@ -399,6 +433,7 @@ __host__ __device__ inline bool secular_root(const Work &w, int lo, int hi, int 
     double lb = o == a ? 0.0 : (last ? 0.0 : w.d[a] - dorg);
     double ub = last ? rho * (1.0 + 0x1p-30) : (o == a ? w.d[b] - dorg : 0.0);  // |z| <= 1 up to rounding
     if (!(x > lb && x < ub)) x = 0.5 * (lb + ub);
+    double prev = INFINITY;
     for (int it = 0; it < kMaxIter; ++it) {
         const Halves<double> h = secular(w, lo, a, hi, c, o, x);
         const double v = irho + h.psi + h.phi;
@@ -408,7 +443,11 @@ __host__ __device__ inline bool secular_root(const Work &w, int lo, int hi, int 
         // rounding level of f at x (Gu & Eisenstat's stopping rule)
         const bool small = fabs(v) <= 0x1p-52 * n * (irho + fabs(h.psi) + fabs(h.phi));
         const double da = (w.d[a] - dorg) - x, db = (w.d[b] - dorg) - x;
-        const double eta = rational_step(h, irho, da, db, v, last);
+        // after a step that left more than a tenth of f, one with the near pole's own weight
+        const bool slow = !(fabs(v) <= 0.1 * prev);
+        prev = fabs(v);
+        const double eta = slow && it > 0 ? fixed_step(h, da, db, v, last, o == a, w.z[o])
+                                          : rational_step(h, da, db, v, last);
         double y = x + eta;
         if (!(y > lb && y < ub)) {
             y = cut(lb, ub);
