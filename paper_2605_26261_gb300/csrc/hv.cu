@@ -291,17 +291,24 @@ ftlm_status launch(const ftlm_basis *b, const V *x, V *y, const EpiDev &ep, int 
     return FTLM_OK;
 }
 
-// Bonds per chunk for 8-wide blocks (FTLM_HV_CHUNK = 2, 4 or 8 overrides the
-// default of 4): a larger chunk keeps more gathers in flight per row, a smaller
-// one leaves registers for more resident warps.
-int chunk8()
+// Bonds per chunk for 8-wide blocks (FTLM_HV_CHUNK = 2, 4 or 8 overrides the choice): a
+// larger chunk keeps more gathers in flight per row, a smaller one leaves registers for
+// more resident warps.  4, but 8 in lookup-table Lanczos launches with few rows, which
+// the resident warps do not fill anyway.  us per launch with 4 and 8, S^z = 0 or 1/2:
+// N = 16 16.6 and 15.7, 18 20.6 and 20.3, 19 26.8 and 24.2, 20 (0.18 M rows) 33.2 and 32.3, 21
+// (0.35 M) 43.2 and 43.3; with combinatorial ranks 19 32.1 and 34.2.  Blocks side by side
+// have grids of their own, so there all CTAs have to fit in the two per SM that chunks
+// of 8 leave (a chain run of N = 18, R = 16 beyond that: 2.64 -> 3.13 ms).
+constexpr uint64_t kChunk8Rows = 1280, kChunk8RowsBlocks = 2 * kRowThreads;  // rows per SM
+
+int chunk8(bool few_rows)
 {
     static const int c = [] {
         const char *e = getenv("FTLM_HV_CHUNK");
         const int v = e ? atoi(e) : 0;
-        return (v == 8 || v == 2) ? v : 4;
+        return (v == 8 || v == 4 || v == 2) ? v : 0;
     }();
-    return c;
+    return c ? c : (few_rows ? 8 : 4);
 }
 
 template <typename V, typename Lbl, bool CLT, bool LANCZOS>
@@ -321,7 +328,8 @@ ftlm_status launch_b(const ftlm_basis *b, int B, const void *x, void *y, const E
     switch (B) {
     case 4: return launch<V, Lbl, CLT, LANCZOS, 1, 4, 8>(b, xv, yv, ep, blocks, stream);
     case 8:
-        switch (chunk8()) {
+        switch (chunk8(CLT && LANCZOS &&
+                       b->D * blocks <= (blocks > 1 ? kChunk8RowsBlocks : kChunk8Rows) * b->num_sms)) {
         case 8: return launch<V, Lbl, CLT, LANCZOS, 1, 8, 8>(b, xv, yv, ep, blocks, stream);
         case 2: return launch<V, Lbl, CLT, LANCZOS, 1, 8, 2>(b, xv, yv, ep, blocks, stream);
         default: return launch<V, Lbl, CLT, LANCZOS, 1, 8, 4>(b, xv, yv, ep, blocks, stream);
