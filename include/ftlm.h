@@ -153,11 +153,11 @@ ftlm_status ftlm_basis_destroy_async(ftlm_basis *basis, void *stream);
  *                     the same 32 columns in the transposed order.
  *   FTLM_HV_AUTO      (default) SPLIT when one block of B vectors of the call
  *                     holds at least 256 MiB (FP32 rows of 32 bytes or more:
- *                     blocks of 8 or 16), 768 MiB (other FP32 blocks) or 1 GiB
- *                     (FP64) and at least
- *                     16 bonds lie inside the high block, else ONE_WALK (the
- *                     crossover measured on GB300; the split moves two row
- *                     streams per step, the one walk misses L2 on long jumps).
+ *                     blocks of 8 or 16) or 768 MiB (other FP32 blocks) and at least
+ *                     16 bonds lie inside the high block, else ONE_WALK, which FP64
+ *                     always takes (the crossover measured on GB300; the split moves two
+ *                     row streams per step, the one walk misses L2 on long jumps; FP64
+ *                     is bound by its arithmetic, of which the one walk has less).
  *   rows_per_tile: high patterns per tile of the transposed walk, 1..32, or 0 for
  *   the default (8).  SPLIT needs 1..64 bonds inside the high block (the N - L
  *   highest sites, L = min(N, 14)); otherwise the sector runs one walk.  Results
@@ -261,8 +261,9 @@ ftlm_status ftlm_lanczos_set_block(int width);
  *   kernel; every chain's arithmetic is its own, so a chain's result does not
  *   depend on the other chains of its block, up to the summation order of the
  *   dot products.  Every sum runs in a fixed order for a given sector, block width
- *   and device, so repeated calls give bit-identical outputs (CR launches hand out
- *   row tiles dynamically, but each tile's sums have a slot of their own).
+ *   and device, so repeated calls give bit-identical outputs (CR and FP32
+ *   general-spin launches hand out row tiles dynamically, but add the tiles' sums as
+ *   whole numbers, whose total does not depend on the order).
  * Outputs (device, row r of chain r, each row M long, entries >= m_eff zero):
  *   theta_dev, weight_dev: double[R*M];  m_eff_dev: int[R];
  *   alpha_dev, beta_dev: double[R*M] or NULL (Lanczos coefficients; beta row r
@@ -477,17 +478,18 @@ void ftlm_flow_destroy(ftlm_flow *flow);
 /* ftlm_ritz -- the Ritz step alone (a5): for each of n chains, the eigenvalues theta
  * and first-component weights w = s_{k,1}^2 of the tridiagonal matrix with diagonal
  * alpha_dev[c*M .. c*M+m-1] and off-diagonal beta_dev[c*M .. c*M+m-2], m = m_dev[c]
- * (0 <= m <= M).  Implicit symmetric QR with Wilkinson shifts in FP64, one thread
- * per chain (up to 32 chains per CTA); outputs ascending, zero past m.  EINVAL for
+ * (0 <= m <= M).  Divide and conquer in FP64, one CTA per chain (implicit symmetric QR with
+ * Wilkinson shifts, one thread per chain, while ftlm_ritz_set_max_sweeps has set a sweep
+ * limit); outputs ascending, zero past m.  EINVAL for
  * n < 0 or M outside 1..FTLM_MAX_LANCZOS. */
 ftlm_status ftlm_ritz(int n, int M, const double *alpha_dev, const double *beta_dev,
                       const int *m_dev, double *theta_dev, double *weight_dev, void *stream);
 
-/* Non-convergence of the tridiagonal eigenproblems.  The implicit QR of the Ritz
- * step (ftlm_ritz, ftlm_lanczos*, ftlm_batch_run) and of the T^(1) spectra of
- * ftlm_ghosts stops after a sweep limit (default 64 m sweeps for an m x m matrix;
- * the Wilkinson shift converges in a few sweeps per eigenvalue).  A chain that
- * reaches the limit gets NaN in its theta and weight rows (ftlm_ghosts: NaN ell,
+/* Non-convergence of the tridiagonal eigenproblems.  The Ritz step (ftlm_ritz,
+ * ftlm_lanczos*, ftlm_batch_run) takes at most 100 steps per root (a few are needed) and
+ * no non-finite coefficient; the implicit QR of the T^(1) spectra of ftlm_ghosts stops
+ * after a sweep limit (default 64 m sweeps for an m x m matrix; the Wilkinson shift
+ * converges in a few sweeps per eigenvalue).  A chain that reaches a limit gets NaN in its theta and weight rows (ftlm_ghosts: NaN ell,
  * no ghost flags), so its NaN propagates into ftlm_thermo's observables, and the
  * device counts it.  Those calls only queue work, so they cannot return the
  * failure themselves:
@@ -496,7 +498,8 @@ ftlm_status ftlm_ritz(int n, int M, const double *alpha_dev, const double *beta_
  *   (work of other streams counts once it has run) in *unconverged (may be NULL),
  *   clears the count, and returns FTLM_ENOCONV when it is not zero.
  * ftlm_ritz_set_max_sweeps -- process-wide sweep limit per problem for later
- *   launches, 0 restores the default (for tests of this path).  EINVAL for < 0. */
+ *   launches, which then run the Ritz step by implicit QR too; 0 restores the default
+ *   (for tests of this path).  EINVAL for < 0. */
 ftlm_status ftlm_ritz_status(void *stream, uint64_t *unconverged);
 ftlm_status ftlm_ritz_set_max_sweeps(int sweeps);
 
