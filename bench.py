@@ -1171,7 +1171,7 @@ def run_serving(args):
                    "admission": "first fit of each sector's units in the flow workspace (32 GB)" +
                                 (f", at most {args.live_rows} rows of flow sectors in flight" if args.live_rows
                                  else ""),
-                   "flow_streams": 4, "small_sectors": "D <= 32768: one persistent batch per job on a side stream",
+                   "flow_streams": 4, "small_sectors": "D <= 32768: one batch per job on a side stream",
                    "l2": "largest sectors (D=10400600, 8 f32 vectors) exceed L2",
                    "parallelism": "single GPU"},
         "p50_ms": sv["p50_ms"], "p99_ms": sv["p99_ms"],

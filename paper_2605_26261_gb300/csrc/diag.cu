@@ -3,7 +3,7 @@
 //
 // Ghosts.  For each chain, T is its m x m Lanczos matrix (theta_k, w_k from the
 // Ritz step) and T^(1) the matrix with the first row and column removed.  Its
-// eigenvalues theta^(1)_j come from the same implicit QR as the Ritz step; with
+// eigenvalues theta^(1)_j come from implicit QR (tridiag.cuh); with
 // both spectra ascending, l_k = min_j |theta_k - theta^(1)_j| (Eq. 25) is found by
 // one merge.  theta_k is a ghost when l_k < tau = C_tau u W_T, W_T = theta_max -
 // theta_min.  Clusters: consecutive ascending theta closer than tau (|theta_k -

@@ -11,12 +11,13 @@
 //  - static tile order (a warp takes every nwarps-th tile of rows): the block sum
 //    is an FP64 tree and the last block to finish adds the per-block partials in
 //    a fixed order and stores alpha_j (epi_end);
-//  - dynamic tile order (CR launches: tiles handed out by a counter, so that all
-//    warps work on one frontier of rows and the gathers of the rows in flight
-//    share L2): each tile's sums go through a fixed warp tree and are added as whole
-//    numbers of two words (AlphaSums), whose sum does not depend on the order; a
-//    launch of one warp turns it into alpha_j.  A slot per tile, added in tile order by
-//    a second launch, cost 15 to 41 us per step and 2 B bytes per row.
+//  - dynamic tile order (CR and FP32 general-spin launches: tiles handed out by a
+//    counter, so that all warps work on one frontier of rows and the gathers of the rows
+//    in flight share L2): each tile's sums go through a fixed warp tree and are added as
+//    whole numbers of two words (AlphaSums), whose sum does not depend on the order; a
+//    launch of one warp (CR) or the last CTA (general spin) turns it into alpha_j.  A
+//    slot per tile, added in tile order by a second launch, cost 15 to 41 us per step and
+//    2 B bytes per row.
 // Either way the result is fixed for a given sector and grid: alpha_j is reproducible.
 #pragma once
 

@@ -11,8 +11,8 @@
 // order, so a unit's results are bit-identical whether it runs alone or with any
 // other units, and whenever it was admitted.  When a unit reaches its last step its
 // chain lengths are copied out; the sectors whose units are all done get their Ritz
-// step, one launch per step call on the flow's own stream (FP64 QR: slow on this
-// GPU, so it overlaps the next call's Lanczos steps instead of delaying them), and
+// step, one launch per step call on the flow's own stream (FP64 work on one SM per
+// chain, so it overlaps the next call's Lanczos steps instead of delaying them), and
 // their coefficient rows are reused once that launch has run.  Units are admitted while their regions fit in the
 // workspace (first fit); a sector that does not fit is refused (FTLM_ENOMEM) and can
 // be added again later.
