@@ -148,6 +148,24 @@ def _stream(stream):
     return ctypes.c_void_p(stream.cuda_stream)
 
 
+def _torch_stream(stream):
+    """`stream` as a torch stream (None: the current one; any object with a cuda_stream
+    handle will do)."""
+    if stream is None:
+        return torch.cuda.current_stream()
+    if isinstance(stream, torch.cuda.Stream):
+        return stream
+    return torch.cuda.ExternalStream(stream.cuda_stream)
+
+
+def _outlive(stream, *tensors):
+    """The tensors' memory is not reused before the work that `stream` holds at the time
+    they are dropped."""
+    for t in tensors:
+        if t is not None and t.is_cuda:
+            t.record_stream(stream)
+
+
 def _ptr(t):
     return None if t is None else ctypes.c_void_p(t.data_ptr())
 
@@ -543,15 +561,7 @@ class Basis:
             pass
 
 
-def lanczos(basis, R, M, seed=1, dist=GAUSS, dtype=torch.float32, start=None, work=None,
-            keep_coeffs=False, stream=None):
-    """Run R chains on one sector; returns dict of device tensors theta, weight
-    (R x M), m_eff (R), and alpha, beta when keep_coeffs."""
-    dev = torch.device("cuda", torch.cuda.current_device())
-    code = _dtype_code(dtype)
-    nbytes = ftlm_lanczos_workspace_bytes(basis.handle, R, M, code)
-    if work is None or work.numel() * work.element_size() < nbytes:
-        work = torch.empty((nbytes + 255) // 256 * 256, dtype=torch.uint8, device=dev)
+def _chain_outputs(R, M, dev, keep_coeffs):
     out = {
         "theta": torch.empty((R, M), dtype=torch.float64, device=dev),
         "weight": torch.empty((R, M), dtype=torch.float64, device=dev),
@@ -560,12 +570,38 @@ def lanczos(basis, R, M, seed=1, dist=GAUSS, dtype=torch.float32, start=None, wo
     if keep_coeffs:
         out["alpha"] = torch.empty((R, M), dtype=torch.float64, device=dev)
         out["beta"] = torch.empty((R, M), dtype=torch.float64, device=dev)
+    return out
+
+
+def lanczos(basis, R, M, seed=1, dist=GAUSS, dtype=torch.float32, start=None, work=None,
+            keep_coeffs=False, stream=None):
+    """Run R chains on one sector; returns dict of device tensors theta, weight
+    (R x M), m_eff (R), and alpha, beta when keep_coeffs."""
+    dev = torch.device("cuda", torch.cuda.current_device())
+    code = _dtype_code(dtype)
+    nbytes = ftlm_lanczos_workspace_bytes(basis.handle, R, M, code)
+    here, on = torch.cuda.current_stream(), _torch_stream(stream)
+    # The call only queues work, and its workspace is dropped on return.  So the memory is
+    # that of the stream the work runs on: whatever takes it next runs after it.
+    away = on.cuda_stream != here.cuda_stream
+    with torch.cuda.stream(on if away else None):
+        held = work
+        if work is None or work.numel() * work.element_size() < nbytes:
+            work = torch.empty((nbytes + 255) // 256 * 256, dtype=torch.uint8, device=dev)
+        out = _chain_outputs(R, M, dev, keep_coeffs)
+    if away:
+        _outlive(here, *out.values())  # the caller may read them there
+        _outlive(on, start, held)
+    _chains(basis, R, M, seed, dist, code, start, work, out, on)
+    return out
+
+
+def _chains(basis, R, M, seed, dist, code, start, work, out, stream):
     args = (work, out["theta"], out["weight"], out["m_eff"], out.get("alpha"), out.get("beta"))
     if start is None:
         ftlm_lanczos(basis.handle, R, M, seed, dist, code, *args, stream=stream)
     else:
         ftlm_lanczos_from(basis.handle, R, M, start, code, *args, stream=stream)
-    return out
 
 
 def thermo(sectors, T, R, M, g=2.0, h=0.0, mirror=True, stream=None):
@@ -769,12 +805,30 @@ def run_ftlm(N, bonds, R, M, T, seed=1, dist=GAUSS, dtype=torch.float32, g=2.0, 
              sectors=None, mode=RANK_AUTO, keep_coeffs=False, stream=None):
     """A whole FTLM job on the device: for each sector (default: every S^z >= 0,
     mirrored), R chains of M steps, then E, C, chi, mag on the grid T.  Everything is
-    queued on `stream` or joined to it; small sectors run side by side."""
-    dev = torch.device("cuda", torch.cuda.current_device())
-    if not torch.is_tensor(T):
-        T = torch.as_tensor(np.asarray(T, dtype=np.float64), device=dev)
-    two = computed_two_sz(N) if sectors is None else list(sectors)
-    base = torch.cuda.current_stream() if stream is None else stream
+    queued on `stream` or joined to it, after the work that the current stream holds
+    (which may still produce T); small sectors run side by side."""
+    here, base = torch.cuda.current_stream(), _torch_stream(stream)
+    away = base.cuda_stream != here.cuda_stream
+    if away:
+        base.wait_stream(here)
+    # Nothing waits for the device before the call returns, so every tensor of the job is
+    # memory of `base`, dropped only once all work on it has been joined to `base`.
+    with torch.cuda.stream(base if away else None):
+        dev = torch.device("cuda", torch.cuda.current_device())
+        if not torch.is_tensor(T):
+            T = torch.as_tensor(np.asarray(T, dtype=np.float64), device=dev)
+        two = computed_two_sz(N) if sectors is None else list(sectors)
+        res = _job_sectors(N, bonds, R, M, seed, dist, dtype, two, mode, keep_coeffs, base, dev)
+        obs = thermo(res, T, R, M, g, h, mirror=sectors is None, stream=base)
+    if away:
+        _outlive(base, T)
+        _outlive(here, *obs.values(), *(t for r in res for t in r[2].values()))
+    obs["sectors"] = res
+    return obs
+
+
+def _job_sectors(N, bonds, R, M, seed, dist, dtype, two, mode, keep_coeffs, base, dev):
+    """The sectors `two` of a job on `base`, the current stream: (two_sz, dim, outputs) each."""
     code = _dtype_code(dtype)
     # a sector's workspace is at least two vectors of its dimension
     row = 2 * (4 if code == F32 else 8)
@@ -793,17 +847,14 @@ def run_ftlm(N, bonds, R, M, T, seed=1, dist=GAUSS, dtype=torch.float32, g=2.0, 
         lanes = [side[i::n] for i in range(n)]
         works = [torch.empty((need[lane[0]] + 255) // 256 * 256, dtype=torch.uint8, device=dev) for lane in lanes]
         by_k = dict(held)
+        for k in side:
+            res[k] = (two[k], by_k[k].dim, _chain_outputs(R, M, dev, keep_coeffs))
         if n > 1:  # the side streams start after the tables, and after this memory's last uses
-            here = torch.cuda.current_stream()
-            for s, w in zip(streams, works):
+            for s in streams:
                 s.wait_stream(base)
-                if here != base:
-                    s.wait_stream(here)
-                w.record_stream(s)
         for lane, s, w in zip(lanes, streams, works):
             for k in lane:
-                res[k] = (two[k], by_k[k].dim,
-                          lanczos(by_k[k], R, M, seed, dist, dtype, work=w, keep_coeffs=keep_coeffs, stream=s))
+                _chains(by_k[k], R, M, seed, dist, code, None, w, res[k][2], s)
         for k, tz in enumerate(two):  # the others one after another on the job's stream
             if res[k] is not None:
                 continue
@@ -822,6 +873,4 @@ def run_ftlm(N, bonds, R, M, T, seed=1, dist=GAUSS, dtype=torch.float32, g=2.0, 
     finally:
         for _, b in held:
             b.release(base)
-    obs = thermo(res, T, R, M, g, h, mirror=sectors is None, stream=base)
-    obs["sectors"] = res
-    return obs
+    return res

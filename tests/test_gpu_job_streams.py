@@ -49,3 +49,30 @@ def test_bad_sector_raises_and_leaves_the_device_usable(cuda_dev):
         assert e.value.status == ftlm.FTLM_EINVAL
     ok = ftlm.run_ftlm(10, inputs.ring(10), 2, 10, T, sectors=[0, 2])
     assert torch.isfinite(ok["E"]).all()
+
+
+@pytest.mark.parametrize("sectors", [[0, 8, 14, 18, 20, 26],  # 10.4 M rows; 3.1 M; 0.23 M and fewer, side by side
+                                     [14],                     # one sector, workspace below SIDE_BYTES
+                                     [8]])                     # one sector, workspace above
+def test_jobs_on_two_streams_without_a_wait(cuda_dev, sectors):
+    N, R, M = 26, 8, 10
+    bonds = inputs.random_graph(N, seed=3)
+    T = torch.logspace(-1, 1, 20, dtype=torch.float64, device=cuda_dev)
+    want = []
+    for seed in (1, 2):
+        want.append(ftlm.run_ftlm(N, bonds, R, M, T, seed=seed, sectors=sectors, keep_coeffs=True))
+        torch.cuda.synchronize()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    got = []
+    for seed, s in zip((1, 2), streams):
+        got.append(ftlm.run_ftlm(N, bonds, R, M, T * 1.0, seed=seed, sectors=sectors, keep_coeffs=True, stream=s))
+        # the caller's next allocations do not share memory with the queued job
+        junk = [torch.full((n << 20,), 255, dtype=torch.uint8, device=cuda_dev) for n in (700, 220, 220, 64, 16, 16, 4)]
+        del junk
+    torch.cuda.synchronize()
+    for g, w in zip(got, want):
+        for k in ("E", "C", "chi", "mag"):
+            assert torch.equal(g[k], w[k]), k
+        for a, b in zip(g["sectors"], w["sectors"]):
+            for k in ("alpha", "beta", "theta", "weight", "m_eff"):
+                assert torch.equal(a[2][k], b[2][k]), (a[0], k)
