@@ -27,6 +27,7 @@
 
 #include "ftlm_internal.cuh"
 #include "reduce.cuh"
+#include "two_word.cuh"
 #include "vec.cuh"
 
 namespace ftlm {
@@ -72,8 +73,8 @@ inline EpiDev epi_of(const LanczosHv *epi)
         ep.counter = epi->counter;
         ep.alpha_out = epi->alpha_out;
         ep.fixed = epi->fixed;
-        // |alpha_j| <= ||H|| < 2^e, and ||y|| <= 2 ||H||: a tile's sum stays below 2^50
-        // units, that of all tiles within 64 bits
+        // |alpha_j| <= ||H|| < 2^e, and ||y|| <= 2 ||H||: the tiles' sums together stay
+        // below 2^50 units in magnitude, whatever their number (two_word.cuh for their rests)
         const int e = epi->norm_bound > 0.0 ? std::ilogb(epi->norm_bound) + 1 : 0;
         const int shift = std::min(1000, 49 - e);
         ep.scale = std::ldexp(1.0, shift);
@@ -179,11 +180,12 @@ __device__ __forceinline__ uint32_t claimed_tile(uint32_t claim, uint32_t nwarps
     return __shfl_sync(0xffffffffu, claim, 0) + nwarps;
 }
 
-// Sums of per-tile values as whole numbers of two words, one pair per warp and chain in
-// shared memory: the first word counts 2^-alpha_shift, the second 2^-(alpha_shift +
+// Sums of per-tile values as whole numbers of two words (two_word.cuh), one pair per warp
+// and chain in shared memory: the first word counts 2^-alpha_shift, the second 2^-(alpha_shift +
 // 40).  Every value is taken to 2^-(alpha_shift + 40), about 2^-90 ||H||, and whole
 // numbers add in any order to the same sum, so the warps may take their tiles in any
-// order.  bad: bit r is set when a value of chain r was not finite.
+// order.  A warp's second word stays below 2^40, so those of all warps of a launch add up
+// within 64 bits.  bad: bit r is set when a value of chain r was not finite.
 template <int B, int THREADS> struct AlphaSums {
     long long v[THREADS / 32][2 * B];
     unsigned int bad;
@@ -205,15 +207,7 @@ __device__ __forceinline__ void add_tile(const EpiDev &ep, AlphaSums<B, THREADS>
     const unsigned lane = threadIdx.x & 31u;
     if (lane < B) {
         const int r = warp_multi_index<B>(lane);
-        long long *w = s.v[threadIdx.x >> 5] + 2 * r;
-        // whole numbers through the mantissa of 1.5 2^52 + v: four FP64 instructions
-        // (conversions to 64-bit integers and back would be four more)
-        constexpr double kOne = 0x1.8p52;
-        const double a = t.value(), m = fma(a, ep.scale, kOne), h = m - kOne;
-        const double f = fma(fma(a, ep.scale, -h), 0x1p40, kOne);
-        if (!(fabs(h) < 0x1p51)) atomicOr(&s.bad, 1u << r);
-        w[0] += __double_as_longlong(m) - __double_as_longlong(kOne);
-        w[1] += __double_as_longlong(f) - __double_as_longlong(kOne);
+        if (!two_word_add(s.v[threadIdx.x >> 5] + 2 * r, t.value(), ep.scale)) atomicOr(&s.bad, 1u << r);
     }
 }
 
@@ -263,7 +257,7 @@ __device__ __forceinline__ void tiles_end(const EpiDev &ep, AlphaSums<B, THREADS
     if (threadIdx.x < B) {
         const int r = threadIdx.x;
         const bool bad = (__ldcg(ep.counter + 3) >> r) & 1u;
-        const double a = ((double)s.v[0][2 * r] + (double)s.v[0][2 * r + 1] * 0x1p-40) * ep.unscale;
+        const double a = two_word_value(s.v[0][2 * r], s.v[0][2 * r + 1], ep.unscale);
         if (!ep.st[r].stopped) {
             ep.st[r].alpha = bad ? NAN : a;
             ep.alpha_out[(size_t)r * ep.alpha_stride] = bad ? NAN : a;

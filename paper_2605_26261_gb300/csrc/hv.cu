@@ -161,7 +161,7 @@ template <int B> __global__ void __launch_bounds__(32) alpha_kernel(const EpiDev
     if (r < B) {
         const long long hi = (long long)ep.fixed[2 * r], lo = (long long)ep.fixed[2 * r + 1];
         const bool bad = (ep.counter[3] >> r) & 1u;
-        const double v = ((double)hi + (double)lo * 0x1p-40) * ep.unscale;
+        const double v = two_word_value(hi, lo, ep.unscale);
         ep.fixed[2 * r] = 0;
         ep.fixed[2 * r + 1] = 0;
         if (!ep.st[r].stopped) {

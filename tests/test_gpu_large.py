@@ -121,3 +121,16 @@ def test_split_lanczos_at_full_size(cuda_dev):
         beta2 = (hq.double() ** 2).sum(dim=0).cpu().numpy() - alpha**2
     np.testing.assert_allclose(a1, alpha, rtol=1e-5, atol=1e-5)
     np.testing.assert_allclose(b1**2, beta2, rtol=1e-4)
+
+
+def test_alpha_of_equal_tile_sums(cuda_dev):
+    """The uniform vector of the N = 32 ring, J = 1.75 (S^z = 0, 601 080 390 rows): 18.8 M tiles
+    with one sum, whose rests in the two-word sums of alpha have one sign and come to
+    1.1 * 2^63.  alpha_1 = N J / 4 to the rounding of a tile's sum (a few 2^-53), and the chain
+    stops at its first step."""
+    with ftlm.Basis(32, 0, inputs.ring(32, 1.75), ftlm.RANK_CR) as b:
+        start = torch.ones((1, b.dim), dtype=torch.float64, device=cuda_dev)
+        out = ftlm.lanczos(b, 1, 3, dtype=torch.float64, start=start, keep_coeffs=True)
+        torch.cuda.synchronize()
+    assert abs(float(out["alpha"][0, 0]) / 14.0 - 1.0) < 1e-14
+    assert int(out["m_eff"][0]) == 1
