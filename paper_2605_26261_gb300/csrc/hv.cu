@@ -240,7 +240,7 @@ bool split_walks(const ftlm_basis *b, int B, size_t vsize, HiWalk *w)
 // One hv_kernel launch over every row.
 template <typename V, typename Lbl, bool CLT, int EPI, int RT, int B, int C>
 ftlm_status launch_rows(const ftlm_basis *b, const BondList &bl, const V *x, V *y, const EpiDev &ep, int blocks,
-                        cudaStream_t stream)
+                        int max_ctas, cudaStream_t stream)
 {
     const size_t smem = CLT ? 0 : ((size_t)1 << b->L) * sizeof(uint16_t);
     auto kern = hv_kernel<V, Lbl, CLT, EPI, RT, B, C>;
@@ -254,7 +254,7 @@ ftlm_status launch_rows(const ftlm_basis *b, const BondList &bl, const V *x, V *
         while (threads > 64 && b->D < (uint64_t)threads * RT * b->num_sms) threads /= 2;
     FTLM_CUDA(kernel_occupancy((const void *)kern, threads, smem_max, false, &occ));
     const uint64_t need = (b->D + (uint64_t)threads * RT - 1) / ((uint64_t)threads * RT);
-    const uint64_t cap = (uint64_t)b->num_sms * std::max(1, std::min({occ, hv_cta_cap(), kMaxBlocksPerSm}));
+    const uint64_t cap = (uint64_t)b->num_sms * std::max(1, std::min({occ, hv_cta_cap(), max_ctas}));
     const int grid = (int)std::max<uint64_t>(1, std::min(need, cap));
     kern<<<dim3(grid, blocks), threads, smem, stream>>>(b->tables(), bl, x, y, ep);
     note_launch();
@@ -262,7 +262,8 @@ ftlm_status launch_rows(const ftlm_basis *b, const BondList &bl, const V *x, V *
 }
 
 template <typename V, typename Lbl, bool CLT, bool LANCZOS, int RT, int B, int C>
-ftlm_status launch(const ftlm_basis *b, const V *x, V *y, const EpiDev &ep, int blocks, cudaStream_t stream)
+ftlm_status launch(const ftlm_basis *b, const V *x, V *y, const EpiDev &ep, int blocks, cudaStream_t stream,
+                   int max_ctas = kMaxBlocksPerSm)
 {
     void *tok = profile_begin(kProfHv, stream, B * blocks);
     ftlm_status st = FTLM_OK;
@@ -277,7 +278,7 @@ ftlm_status launch(const ftlm_basis *b, const V *x, V *y, const EpiDev &ep, int 
                                        : fail(FTLM_EUNSUPPORTED, "split H.v without a walk A tile table");
             if (st == FTLM_OK) st = launch_walk_b(b, w, dt, B, x, y, ep, stream);
         } else {
-            st = launch_rows<V, Lbl, false, kLanczos, RT, B, C>(b, b->bonds_cr, x, y, ep, blocks, stream);
+            st = launch_rows<V, Lbl, false, kLanczos, RT, B, C>(b, b->bonds_cr, x, y, ep, blocks, max_ctas, stream);
         }
         if (st == FTLM_OK) {
             alpha_kernel<B><<<dim3(1, blocks), 32, 0, stream>>>(ep);
@@ -285,7 +286,7 @@ ftlm_status launch(const ftlm_basis *b, const V *x, V *y, const EpiDev &ep, int 
         }
     } else {
         st = launch_rows<V, Lbl, CLT, LANCZOS ? kLanczos : kPlain, RT, B, C>(b, CLT ? b->bonds_clt : b->bonds_cr, x,
-                                                                           y, ep, blocks, stream);
+                                                                           y, ep, blocks, max_ctas, stream);
     }
     profile_end(tok, stream);
     if (st != FTLM_OK) return st;
@@ -298,19 +299,28 @@ ftlm_status launch(const ftlm_basis *b, const V *x, V *y, const EpiDev &ep, int 
 // more resident warps.  4, but 8 in lookup-table Lanczos launches with few rows, which
 // the resident warps do not fill anyway.  us per launch with 4 and 8, S^z = 0 or 1/2:
 // N = 16 16.6 and 15.7, 18 20.6 and 20.3, 19 26.8 and 24.2, 20 (0.18 M rows) 33.2 and 32.3, 21
-// (0.35 M) 43.2 and 43.3; with combinatorial ranks 19 32.1 and 34.2.  Blocks side by side
-// have grids of their own, so there all CTAs have to fit in the two per SM that chunks
-// of 8 leave (a chain run of N = 18, R = 16 beyond that: 2.64 -> 3.13 ms).
-constexpr uint64_t kChunk8Rows = 1280, kChunk8RowsBlocks = 2 * kRowThreads;  // rows per SM
+// (0.35 M) 43.2 and 43.3; with combinatorial ranks 19 32.1 and 34.2.
+//
+// Blocks side by side have a grid each.  A block's grid fixes the order of its sums, so it is
+// that of chunks of 8 (two CTAs per SM) for every sector of few rows, whichever chunk the
+// launch takes; the chunk changes no result.  Chunks of 8 there while all CTAs fit in two per
+// SM, and from the rows where a block alone fills those twice; between the two chunks of
+// 4.  ms per run of 100 steps, two blocks, chunks of 4 and 8 (and 4 with the grid of three
+// CTAs per SM that a block alone does not have): 320 rows per SM 4.46 and 5.23 (4.45), 608
+// 6.29 and 6.39 (6.67), 829 7.43 and 7.10 (7.81), 1105 9.08 and 8.53 (8.31), 1215 8.76 and 8.56
+// (8.65); three blocks 608 8.05 and 8.62 (9.05), 829 9.30 and 9.70 (10.28), 1105 13.8 and 13.3
+// (13.1), 1215 13.8 and 13.5 (13.7).
+constexpr uint64_t kChunk8Rows = 1280, kChunk8RowsBlocks = 2 * kRowThreads,
+                   kChunk8RowsFull = 4 * kRowThreads;  // rows per SM
 
-int chunk8(bool few_rows)
+int chunk8(bool wide)
 {
     static const int c = [] {
         const char *e = getenv("FTLM_HV_CHUNK");
         const int v = e ? atoi(e) : 0;
         return (v == 8 || v == 4 || v == 2) ? v : 0;
     }();
-    return c ? c : (few_rows ? 8 : 4);
+    return c ? c : (wide ? 8 : 4);
 }
 
 template <typename V, typename Lbl, bool CLT, bool LANCZOS>
@@ -329,13 +339,17 @@ ftlm_status launch_b(const ftlm_basis *b, int B, const void *x, void *y, const E
     } else {
     switch (B) {
     case 4: return launch<V, Lbl, CLT, LANCZOS, 1, 4, 8>(b, xv, yv, ep, blocks, stream);
-    case 8:
-        switch (chunk8(CLT && LANCZOS &&
-                       b->D * blocks <= (blocks > 1 ? kChunk8RowsBlocks : kChunk8Rows) * b->num_sms)) {
-        case 8: return launch<V, Lbl, CLT, LANCZOS, 1, 8, 8>(b, xv, yv, ep, blocks, stream);
-        case 2: return launch<V, Lbl, CLT, LANCZOS, 1, 8, 2>(b, xv, yv, ep, blocks, stream);
-        default: return launch<V, Lbl, CLT, LANCZOS, 1, 8, 4>(b, xv, yv, ep, blocks, stream);
+    case 8: {
+        const bool few = CLT && LANCZOS && b->D <= kChunk8Rows * b->num_sms;
+        const int ctas = few ? min_ctas<V, 1, 8, 8>() : kMaxBlocksPerSm;
+        const bool wide = blocks == 1 || b->D * blocks <= kChunk8RowsBlocks * b->num_sms ||
+                          b->D >= kChunk8RowsFull * b->num_sms;
+        switch (chunk8(few && wide)) {
+        case 8: return launch<V, Lbl, CLT, LANCZOS, 1, 8, 8>(b, xv, yv, ep, blocks, stream, ctas);
+        case 2: return launch<V, Lbl, CLT, LANCZOS, 1, 8, 2>(b, xv, yv, ep, blocks, stream, ctas);
+        default: return launch<V, Lbl, CLT, LANCZOS, 1, 8, 4>(b, xv, yv, ep, blocks, stream, ctas);
         }
+    }
     case 16: return launch<V, Lbl, CLT, LANCZOS, 1, 16, 4>(b, xv, yv, ep, blocks, stream);
     default: break;
     }

@@ -45,3 +45,17 @@ def test_workspace_keeps_the_scratch_free_limit(cuda_dev):
             many = ftlm.ftlm_lanczos_workspace_bytes(b.handle, R, 20, torch.float32)
             assert many >= one
             assert many <= max(24 << 20, 10 * one)
+
+
+@pytest.mark.parametrize("N,R", [(18, 16), (19, 16), (19, 24), (20, 16), (20, 24), (21, 24)])
+def test_a_chain_does_not_depend_on_the_blocks_beside_it(cuda_dev, N, R):
+    # around the row counts where the H.v launch changes its shape: 320, 608, 1215 and 2320 rows per
+    # SM, with two and three blocks of 8 side by side, or two and then one, where they fit
+    with ftlm.Basis(N, N % 2, inputs.random_graph(N, seed=4), ftlm.RANK_CLT) as b:
+        g = torch.Generator(device=cuda_dev).manual_seed(3)
+        start = torch.randn((R, b.dim), generator=g, device=cuda_dev, dtype=torch.float64)
+        whole = ftlm.lanczos(b, R, 9, dtype=torch.float32, start=start, keep_coeffs=True)
+        for r in range(0, R, 8):
+            part = ftlm.lanczos(b, 8, 9, dtype=torch.float32, start=start[r:r + 8].contiguous(), keep_coeffs=True)
+            for k in ("alpha", "beta", "theta", "weight", "m_eff"):
+                assert torch.equal(whole[k][r:r + 8], part[k]), (k, r)
