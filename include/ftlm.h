@@ -384,10 +384,11 @@ ftlm_status ftlm_batch_destroy_async(ftlm_batch *batch, void *stream);
  * 2^20; 0: 2048, and D / 32 between 2048 and 16384).  ftlm_batch_create_plan plans with them (results agree
  * with other plans up to the summation order of the per-tile sums).
  * ftlm_batch_autotune_plan times candidate plans on the items (each candidate: one
- * untimed and one timed run, as ftlm_batch_autotune) by coordinate search -- block
- * width in {4, 8, 16} (and side streams in {1, 2, 4, 8} when an item runs on
- * them), then tile_rows in {1024, 2048, 4096} and stream_rows in {8192, 16384,
- * 32768} when an item runs on the multi-sector path -- and returns the fastest in
+ * untimed and one timed run, as ftlm_batch_autotune) by coordinate search from the
+ * default plan -- block width in {4, 8, 16} (and side streams in {1, 2, 4, 8} when an
+ * item runs on them), then, when an item runs on the multi-sector path, tile_rows of 1024
+ * and 4096 with stream_rows of 8192 and 32768, and stream_rows of 16384 and 32768 (0
+ * if it is set by then) alone -- and returns the fastest in
  * *best; the first max_tried candidates and their times go to tried / ms_out,
  * *n_tried = candidates timed.  Blocks the host; overwrites the items' outputs. */
 typedef struct {

@@ -891,12 +891,16 @@ extern "C" ftlm_status ftlm_batch_autotune_plan(int n, const ftlm_batch_item *it
     cudaEvent_t ev[2] = {nullptr, nullptr};
     FTLM_CUDA(cudaEventCreate(&ev[0]));
     FTLM_CUDA(cudaEventCreate(&ev[1]));
-    ftlm_batch_plan cur{8, any_large ? 4 : 1, (int)kMsTileRows, (int)kMsStreamRows};
+    ftlm_batch_plan cur{8, any_large ? 4 : 1, (int)kMsTileRows, 0};
     float cur_ms = -1.f;
     int count = 0;
     ftlm_status st = FTLM_OK;
-    // coordinate search: block width (with the side-stream count where it matters),
-    // then the H.v tile rows and the streaming tile rows of the multi-sector path
+    // coordinate search from the plan that ftlm_batch_create makes: block width (with the
+    // side-stream count where it matters), then the H.v tiles of the multi-sector path, with
+    // streaming tiles of eight of them, then the streaming tiles alone.  stream_rows = 0 (by
+    // the sector's rows) is among the candidates: one number of rows suits no batch of
+    // sectors of different sizes (13 sectors of the spin-1 icosahedron 17.2 ms with 16384 rows, 15.2
+    // with 0).
     auto consider = [&](const ftlm_batch_plan &cand) {
         float ms = 0.f;
         st = time_plan(n, items, M, dist, dtype, cand, stream, pool, ev, &ms);
@@ -921,14 +925,15 @@ extern "C" ftlm_status ftlm_batch_autotune_plan(int n, const ftlm_batch_item *it
         }
     if (any_ms) {
         const ftlm_batch_plan base = cur;
-        for (int tr : {1024, 4096}) {
+        for (int tr : {(int)kMsTileRows / 2, (int)kMsTileRows * 2}) {
             if (st != FTLM_OK) break;
             ftlm_batch_plan c = base;
             c.tile_rows = tr;
+            c.stream_rows = 8 * tr;
             consider(c);
         }
         const ftlm_batch_plan base2 = cur;
-        for (int sr : {8192, 32768}) {
+        for (int sr : {(int)kMsStreamRows, base2.stream_rows ? 0 : 2 * (int)kMsStreamRows}) {
             if (st != FTLM_OK) break;
             ftlm_batch_plan c = base2;
             c.stream_rows = sr;

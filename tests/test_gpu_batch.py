@@ -326,3 +326,16 @@ def test_plan_autotune_tunes_tiles_and_plans_agree(cuda_dev):
         ftlm.Batch(entries, M, ftlm.GAUSS, torch.float32, plan=ftlm.BatchPlan(8, 1, 1000, 0))
     for b in bases:
         b.close()
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+def test_plan_autotune_times_the_default_plan(cuda_dev, dtype):
+    bases = _mid_sector_bases()
+    entries = [(b, 8, 1, 0) for b in bases]
+    best, tried = ftlm.autotune_plan(entries, 15, ftlm.GAUSS, dtype)
+    times = dict(tried)
+    assert (8, 1, 2048, 0) in times  # blocks of 8, tiles by the sector's rows: what ftlm_batch_create plans
+    assert times[best.as_tuple()] <= times[(8, 1, 2048, 0)]
+    assert len(times) == len(tried)  # no candidate twice
+    for b in bases:
+        b.close()
