@@ -799,6 +799,10 @@ def computed_two_sz(N, two_s=1):
 # microseconds each on a part of the SMs (N = 16 ring, FP64, R = 20, nine sectors:
 # 28.2 ms one after another).
 SIDE_BYTES, SIDE_STREAMS = 64 << 20, 4
+# They run in groups whose tables take at most this much together (a lookup table is 2^N / 4
+# bytes, however few rows the sector has: all 13 of N = 26 are 0.2 GB, one of N = 32
+# 1.1 GB), and no table is held under the larger sectors' chains.
+TABLE_BYTES = 1 << 30
 
 
 def run_ftlm(N, bonds, R, M, T, seed=1, dist=GAUSS, dtype=torch.float32, g=2.0, h=0.0,
@@ -829,48 +833,58 @@ def run_ftlm(N, bonds, R, M, T, seed=1, dist=GAUSS, dtype=torch.float32, g=2.0, 
 
 def _job_sectors(N, bonds, R, M, seed, dist, dtype, two, mode, keep_coeffs, base, dev):
     """The sectors `two` of a job on `base`, the current stream: (two_sz, dim, outputs) each."""
-    code = _dtype_code(dtype)
     # a sector's workspace is at least two vectors of its dimension
-    row = 2 * (4 if code == F32 else 8)
+    row = 2 * (4 if _dtype_code(dtype) == F32 else 8)
     small = [k for k, tz in enumerate(two)
              if abs(tz) <= N and math.comb(int(N), (int(N) + int(tz)) // 2) * row <= SIDE_BYTES]
+    chains = (R, M, seed, dist, dtype, keep_coeffs, base)
     res = [None] * len(two)
-    held = []
+    # bytes of a sector's tables at most: 2^N / 4 of a lookup table (N <= 32), 2^N / 1024 of ranks by digit blocks
+    table = (1 << max(0, N - 2 if N <= 32 else N - 10)) + (4 << 20) if small else 1
+    size = max(1, min(MAX_SECTORS, TABLE_BYTES // table))
+    group = {}  # sectors whose tables are held
     try:
-        for a in range(0, len(small), MAX_SECTORS):
-            ks = small[a:a + MAX_SECTORS]
-            held += zip(ks, Basis.sectors(N, [two[k] for k in ks], bonds, mode, base, wait=False))
-        need = {k: ftlm_lanczos_workspace_bytes(b.handle, R, M, code) for k, b in held}
-        side = sorted((k for k, _ in held if need[k] <= SIDE_BYTES), key=lambda k: -need[k])
-        n = min(SIDE_STREAMS, len(side))
-        streams = [torch.cuda.Stream(dev) for _ in range(n)] if n > 1 else [base] * n
-        lanes = [side[i::n] for i in range(n)]
-        works = [torch.empty((need[lane[0]] + 255) // 256 * 256, dtype=torch.uint8, device=dev) for lane in lanes]
-        by_k = dict(held)
-        for k in side:
-            res[k] = (two[k], by_k[k].dim, _chain_outputs(R, M, dev, keep_coeffs))
-        if n > 1:  # the side streams start after the tables, and after this memory's last uses
-            for s in streams:
-                s.wait_stream(base)
-        for lane, s, w in zip(lanes, streams, works):
-            for k in lane:
-                _chains(by_k[k], R, M, seed, dist, code, None, w, res[k][2], s)
-        for k, tz in enumerate(two):  # the others one after another on the job's stream
-            if res[k] is not None:
-                continue
-            if k in by_k:
-                res[k] = (tz, by_k[k].dim,
-                          lanczos(by_k[k], R, M, seed, dist, dtype, keep_coeffs=keep_coeffs, stream=base))
-                continue
-            with Basis(N, tz, bonds, mode, base) as b:
-                res[k] = (tz, b.dim, lanczos(b, R, M, seed, dist, dtype, keep_coeffs=keep_coeffs, stream=base))
-        if n > 1:
-            for s in streams:
-                base.wait_stream(s)
+        for a in range(0, len(small), size):
+            ks = small[a:a + size]
+            group = dict(zip(ks, Basis.sectors(N, [two[k] for k in ks], bonds, mode, base, wait=False)))
+            _group_sectors(group, two, res, chains, dev)
+        for k, tz in enumerate(two):  # the others one after another
+            if res[k] is None:
+                with Basis(N, tz, bonds, mode, base) as b:
+                    res[k] = (tz, b.dim, lanczos(b, R, M, seed, dist, dtype, keep_coeffs=keep_coeffs, stream=base))
     except BaseException:
         torch.cuda.synchronize(dev)  # side work may still use the tables and workspaces
         raise
     finally:
-        for _, b in held:
+        for b in group.values():
             b.release(base)
     return res
+
+
+def _group_sectors(group, two, res, chains, dev):
+    """The sectors of `group` (k: Basis): those with small workspaces over side streams, the
+    others on the job's stream beside them.  Releases the tables in that stream's order."""
+    R, M, seed, dist, dtype, keep_coeffs, base = chains
+    code = _dtype_code(dtype)
+    need = {k: ftlm_lanczos_workspace_bytes(b.handle, R, M, code) for k, b in group.items()}
+    side = sorted((k for k in group if need[k] <= SIDE_BYTES), key=lambda k: -need[k])
+    n = min(SIDE_STREAMS, len(side))
+    streams = [torch.cuda.Stream(dev) for _ in range(n)] if n > 1 else [base] * n
+    lanes = [side[i::n] for i in range(n)]
+    works = [torch.empty((need[lane[0]] + 255) // 256 * 256, dtype=torch.uint8, device=dev) for lane in lanes]
+    for k in side:
+        res[k] = (two[k], group[k].dim, _chain_outputs(R, M, dev, keep_coeffs))
+    if n > 1:  # the side streams start after the tables, and after this memory's last uses
+        for s in streams:
+            s.wait_stream(base)
+    for lane, s, w in zip(lanes, streams, works):
+        for k in lane:
+            _chains(group[k], R, M, seed, dist, code, None, w, res[k][2], s)
+    for k, b in group.items():
+        if need[k] > SIDE_BYTES:
+            res[k] = (two[k], b.dim, lanczos(b, R, M, seed, dist, dtype, keep_coeffs=keep_coeffs, stream=base))
+    if n > 1:
+        for s in streams:
+            base.wait_stream(s)
+    for b in group.values():
+        b.release(base)

@@ -8,6 +8,7 @@ drop is checked against the allocator's contract:
   - a use on another stream has to come after the owner's earlier work (the block's last
     owner), and after the writes it reads.
 """
+import math
 import types
 
 import numpy as np
@@ -20,6 +21,8 @@ from paper_2605_26261_gb300 import ftlm
 class World:
     def __init__(self):
         self.errors, self.done, self.count = [], {}, 0
+        self.held, self.peak, self.built = 0, 0, []  # bytes of tables now and at most; (sector, bytes held before it)
+        self.tables = lambda N, two_sz: 1 << 20
         Stream.world, Stream.clocks = self, {}
         self.here = Stream()
         self.current = self.here
@@ -118,7 +121,11 @@ def make(monkeypatch, needs):
 
     class Basis:
         def __init__(self, N, two_sz, bonds, mode=0, stream=None, wait=True):
-            self.two_sz, self.handle, self.dim, self.table_bytes = two_sz, self, 100, 1 << 20
+            self.two_sz, self.handle, self.dim = two_sz, self, 100
+            self.table_bytes = w.tables(N, two_sz)
+            w.held += self.table_bytes
+            w.peak = max(w.peak, w.held)
+            w.built.append((two_sz, w.held - self.table_bytes))
             self.table = w.tensor((1,))
             self.table.owner = stream
             self.table.use(stream, stream.op(), "tables", write=True)
@@ -130,10 +137,13 @@ def make(monkeypatch, needs):
             return [cls(N, tz, bonds, mode, stream, wait) for tz in two_sz]
 
         def release(self, stream):
-            self.table.owner, self.table = stream, None
+            if self.table:
+                w.held -= self.table_bytes
+                self.table.owner, self.table = stream, None
 
         def close(self):
             w.synchronize()
+            w.held -= self.table_bytes
             self.table = None
 
         def __enter__(self):
@@ -240,3 +250,20 @@ def test_any_object_with_a_stream_handle(monkeypatch):
     ftlm.torch.cuda.ExternalStream = external
     ftlm.run_ftlm(30, ((), (), ()), 8, 10, np.ones(4), sectors=[20, 22], stream=types.SimpleNamespace(cuda_stream=77))
     assert set(wrapped) == {77} and w.errors == []
+
+
+@pytest.mark.parametrize("N", [20, 26, 28, 30, 32])
+def test_tables_held_at_once(monkeypatch, N):
+    """All sectors of a job: the tables held at once stay within TABLE_BYTES (one sector's where
+    that is larger), and none is held when a large sector's chains start."""
+    two = ftlm.computed_two_sz(N)
+    dims = {tz: math.comb(N, (N + tz) // 2) for tz in two}
+    w = make(monkeypatch, {tz: 2 * 8 * 4 * d for tz, d in dims.items()})
+    lookup = (1 << N) // 4
+    w.tables = lambda N, tz: lookup + 4 * dims[tz] if dims[tz] < 1 << 20 else 1 << 18
+    ftlm.run_ftlm(N, ((), (), ()), 8, 10, np.ones(4))
+    assert w.errors == [] and w.held == 0 and len(w.built) == len(two)
+    assert w.peak <= max(ftlm.TABLE_BYTES + lookup, w.tables(N, two[-1]) + (1 << 23))
+    for tz, held in w.built:
+        if 8 * dims[tz] > ftlm.SIDE_BYTES:
+            assert held == 0, tz
