@@ -224,11 +224,10 @@ ftlm_status ftlm_hv_block(const ftlm_basis *basis, ftlm_dtype dtype, int B, cons
 
 /* ---------------------------------------------------------------- Lanczos ---
  * Workspace bytes ftlm_lanczos / ftlm_lanczos_from need for R chains of at most M
- * steps: two blocks of D x B_w elements of dtype plus O(R M) coefficients, and for
- * CR spin-1/2 sectors ceil(D / 32) x B_w doubles for the dot-product sums; B_w
- * is the widest block of chains (chains go in blocks of 16, 8 or 4 interleaved
- * vectors, up to the width of ftlm_lanczos_set_block -- by default 8 in FP32 and 4
- * in FP64 -- then single chains).  Blocks of one width run side by side, each with
+ * steps: two blocks of D x B_w elements of dtype plus O(R M) coefficients and the
+ * partial sums of the launches (B_w doubles per CTA); B_w is the widest block of
+ * chains (chains go in blocks of 16, 8 or 4 interleaved vectors, up to the width of
+ * ftlm_lanczos_set_block -- by default 8 in FP32 and 4 in FP64 -- then single chains).  Blocks of one width run side by side, each with
  * its own vectors and sums, as far as the whole workspace stays within 24 MiB.  EINVAL for R < 1 or M
  * outside 1..FTLM_MAX_LANCZOS. */
 ftlm_status ftlm_lanczos_workspace_bytes(const ftlm_basis *basis, int R, int M, ftlm_dtype dtype,

@@ -286,10 +286,6 @@ bool valid_block(int B);
 bool hv_splits(const ftlm_basis *b, ftlm_dtype dtype, int B);
 // FTLM_RANK_AUTO picks CR for sectors of at least this many rows.
 constexpr uint64_t kAutoCrRows = 1ull << 20;
-// Upper bound on the tiles of a Lanczos H.v launch of B vectors that takes its tiles
-// in dynamic order (CR rank mode, one walk or split), at least one; 0 for the others.
-// The workspace has B doubles per tile for it.
-uint32_t hv_lanczos_tiles(const ftlm_basis *b, int B);
 
 // ---- split Lanczos H.v (basis.cu, walkb.cu, hv.cu) -------------------------
 // Walk B's tile layout for rh high patterns per tile (1 <= rh <= 32); false when

@@ -389,16 +389,6 @@ bool hv_splits(const ftlm_basis *b, ftlm_dtype dtype, int B)
     return b->two_s == 1 && b->mode == FTLM_RANK_CR && split_walks(b, B, dtype == FTLM_F32 ? 4 : 8, &w);
 }
 
-uint32_t hv_lanczos_tiles(const ftlm_basis *b, int B)
-{
-    if (b->two_s > 1 || b->mode == FTLM_RANK_CLT) return 0;
-    const uint64_t rows = 32ull * (B == 1 ? rows_per_thread(false) : 1);  // FP32; rows of doubles take 32
-    uint32_t n = (uint32_t)((b->D + rows - 1) / rows);
-    HiWalk w;  // walk B has the most tiles with one high pattern per tile
-    if (build_hi_walk(b, 1, &w)) n = std::max(n, w.ntiles);
-    return n;
-}
-
 ftlm_status launch_hv(const ftlm_basis *b, ftlm_dtype dtype, int B, const void *x, void *y,
                       const LanczosHv *epi, cudaStream_t stream)
 {

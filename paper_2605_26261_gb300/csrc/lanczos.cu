@@ -440,12 +440,11 @@ std::vector<int> block_plan(int R, ftlm_dtype dtype, int bmax)
 constexpr uint64_t kSideBySideBytes = 24ull << 20;
 
 // Workspace: `slots` block slots (two vector blocks, partials, states and counters, and
-// the alpha sums of dynamically ordered H.v launches, of which kAlphaFixedBytes are
-// used), then the coefficients of every chain.
+// the alpha sums of CR H.v launches), then the coefficients of every chain.
 struct Layout {
     int bw;     // widest block
     int slots;  // blocks side by side
-    uint64_t slot, vec1, partials, state, tiles;  // bytes of a slot and offsets in it (vectors first)
+    uint64_t slot, vec1, partials, state, sums;  // bytes of a slot and offsets in it (vectors first)
     uint64_t alpha, beta, meff, total;
 };
 
@@ -464,8 +463,8 @@ Layout layout(const ftlm_basis *b, int R, int M, ftlm_dtype dtype, int bmax = 0)
     l.vec1 = vb;
     l.partials = 2 * vb;
     l.state = l.partials + align256((uint64_t)max_row_grid(b) * l.bw * sizeof(double));
-    l.tiles = l.state + align256(l.bw * sizeof(ChainState) + 64);
-    l.slot = l.tiles + align256((uint64_t)hv_lanczos_tiles(b, 4) * l.bw * sizeof(double));
+    l.sums = l.state + align256(l.bw * sizeof(ChainState) + 64);
+    l.slot = l.sums + (b->two_s == 1 && b->mode == FTLM_RANK_CR ? align256(kAlphaFixedBytes) : 0);
     const uint64_t rows = 2 * align256((uint64_t)R * M * sizeof(double)) + align256((uint64_t)R * sizeof(int));
     const uint64_t room = kSideBySideBytes > rows ? kSideBySideBytes - rows : 0;
     l.slots = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)most, room / l.slot));
@@ -502,8 +501,7 @@ ftlm_status run_blocks(const ftlm_basis *b, int M, int r0, int n, int chain0, ui
     const BlockSlots slots{lay.slot};
 
     // states and counters, and the alpha sums behind them
-    const uint64_t zero = lay.slot > lay.tiles ? lay.tiles - lay.state + kAlphaFixedBytes
-                                               : lay.bw * sizeof(ChainState) + 64;
+    const uint64_t zero = lay.slot > lay.sums ? lay.slot - lay.state : lay.bw * sizeof(ChainState) + 64;
     FTLM_CUDA(cudaMemset2DAsync(st, lay.slot, 0, zero, n, stream));
     start_kernel<V, B><<<g_start, kRowThreads, 0, stream>>>(
         D, KeySpec{seed, b->key_n, b->K, chain0 + r0}, dist, src ? src + (size_t)r0 * D : nullptr, vec[0], st,
@@ -513,7 +511,7 @@ ftlm_status run_blocks(const ftlm_basis *b, int M, int r0, int n, int chain0, ui
     int cur = 0;
     for (int j = 1; j <= m_max; ++j) {
         LanczosHv epi{st, partials, counter, alpha_ws + (size_t)r0 * M + (j - 1), M, j,
-                      (unsigned long long *)(ws + lay.tiles), b->tau64 * (0x1p53 / 100.0), n, lay.slot};
+                      (unsigned long long *)(ws + lay.sums), b->tau64 * (0x1p53 / 100.0), n, lay.slot};
         ftlm_status s = launch_hv(b, dtype, B, vec[cur], vec[1 - cur], &epi, stream);
         if (s != FTLM_OK) return s;
         void *tok = profile_begin(kProfUpdate, stream);

@@ -59,3 +59,13 @@ def test_a_chain_does_not_depend_on_the_blocks_beside_it(cuda_dev, N, R):
             part = ftlm.lanczos(b, 8, 9, dtype=torch.float32, start=start[r:r + 8].contiguous(), keep_coeffs=True)
             for k in ("alpha", "beta", "theta", "weight", "m_eff"):
                 assert torch.equal(whole[k][r:r + 8], part[k]), (k, r)
+
+
+@pytest.mark.parametrize("mode", [ftlm.RANK_CLT, ftlm.RANK_CR])
+@pytest.mark.parametrize("N,R,width", [(22, 8, 8), (23, 9, 8), (23, 1, 1), (24, 4, 4)])
+def test_workspace_is_two_vector_blocks(cuda_dev, mode, N, R, width):
+    with ftlm.Basis(N, N % 2, inputs.ring(N), mode) as b:
+        for dtype, size in ((torch.float32, 4), (torch.float64, 8)):
+            vectors = 2 * b.dim * min(width, 32 // size) * size  # blocks of 8 floats, 4 doubles
+            got = ftlm.ftlm_lanczos_workspace_bytes(b.handle, R, 50, dtype)
+            assert vectors <= got <= max(24 << 20, vectors + (1 << 18))
