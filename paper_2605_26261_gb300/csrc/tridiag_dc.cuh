@@ -17,12 +17,12 @@
 //
 // Bound: FP64 instructions (two lanes per cycle and SM).  Per root of a merge of n
 // poles four passes over the poles remain: a float estimate (not on the FP64 pipe)
-// leaves two double steps, then z and the rows take one pass each, about 33 FP64
+// leaves two double steps, then z and the rows take one pass each, about 37 FP64
 // instructions per pole and root; the merges of all levels cost twice the last one.
 // Measured on GB300, rows of Lanczos coefficients, against implicit QR with one thread
 // per problem (a chain of about m^2 dependent rotations), n problems of m rows: m = 100,
-// n = 8 / 690 / 4096: 21.2 / 21.3 / 21.3 ms -> 0.53 / 1.5 / 8.4 ms; m = 20, n = 8: 0.97
-// -> 0.15 ms; m = 300, n = 8: 180 -> 4.8 ms; only for tens of thousands of problems at
+// n = 8 / 690 / 4096: 21.2 / 21.3 / 21.3 ms -> 0.56 / 1.7 / 9.0 ms; m = 20, n = 8: 0.97
+// -> 0.15 ms; m = 300, n = 8: 180 -> 5.1 ms; only for tens of thousands of problems at
 // once is QR as fast.  Without the float estimate (doubles from the middle of the gap)
 // 1.6 ms at m = 100, n = 8; with the half-sum steps alone 0.96 ms, 10 to 18 double steps for
 // one or two roots of the last merge.
@@ -71,16 +71,18 @@ __host__ __device__ inline Work carve(void *p, int m)
     return w;
 }
 
-// 1 / x to working accuracy without the special cases of a division: the hardware's
-// approximation (relative error below 2^-20) and one third-order correction, error
-// 2^-60 before rounding.  Zero and infinite results need not be finite here.
+// 1 / x within one unit in the last place for 2^-1021 <= |x| <= 2^1021 (NaN for subnormal x and zero):
+// the Newton-Raphson iteration r (2 - x r) for the reciprocal, two steps from the PTX ISA's
+// rcp.approx.ftz.f64, whose error of about 2^-20 they square twice.  No branch and four FP64
+// instructions; with 1.0 / x the Ritz step of 8 / 690 chains of m = 100 takes 0.60 / 2.50 ms
+// instead of 0.56 / 1.66.
 __host__ __device__ __forceinline__ double recip(double x)
 {
 #ifdef __CUDA_ARCH__
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    const double e = fma(-x, r, 1.0);
-    return fma(r, fma(e, e, e), r);
+    r = fma(r, fma(-x, r, 1.0), r);
+    return fma(r, fma(-x, r, 1.0), r);
 #else
     return 1.0 / x;
 #endif

@@ -7,6 +7,9 @@ of 2^-52 ||T|| (1e-13: 450 of them), and so are the smooth spectral sums
 sum_k w_k g(theta_k) with |g|, |g'| ||T|| <= 8 (1e-12).  Weights inside a cluster of
 close eigenvalues are defined only as a sum, hence the sums.
 """
+import ctypes
+import subprocess
+
 import numpy as np
 import pytest
 import torch
@@ -95,3 +98,47 @@ def test_a_chain_does_not_depend_on_the_others(cuda_dev):
     for c in (0, 17, 39):
         t1, w1 = ritz(a[c:c + 1], b[c:c + 1], m[c:c + 1], cuda_dev)
         assert np.array_equal(t1[0], th[c]) and np.array_equal(w1[0], w[c])
+
+
+RECIP = r"""
+#include <cstring>
+#include "tridiag_dc.cuh"
+__global__ void recip_kernel(int n, const double *x, double *got, double *want)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) {
+        got[i] = ftlm::dc::recip(x[i]);
+        want[i] = __drcp_rn(x[i]);
+    }
+}
+extern "C" int recip_all(int n, const double *x, double *got, double *want)
+{
+    recip_kernel<<<(n + 255) / 256, 256>>>(n, x, got, want);
+    return (int)cudaDeviceSynchronize();
+}
+"""
+
+
+def test_reciprocal_against_cuda(cuda_dev, tmp_path):
+    """dc::recip against the correctly rounded reciprocal over its range: within one unit in the last
+    place (the Newton step's own rounding is half of one; the error before it is 2^-80)."""
+    from paper_2605_26261_gb300 import _build
+
+    src, so = tmp_path / "recip.cu", tmp_path / "recip.so"
+    src.write_text(RECIP)
+    subprocess.run([_build._nvcc(), "-shared", "-Xcompiler", "-fPIC", "-std=c++17", *_build.ARCH, "-I", _build.CSRC,
+                    str(src), "-o", str(so)], check=True)
+    rng = np.random.default_rng(5)
+    n = 1 << 20
+    x = np.ldexp(1.0 + rng.random(n), rng.integers(-1021, 1021, size=n)) * rng.choice([-1.0, 1.0], size=n)
+    x[:n // 2] = np.ldexp(1.0 + rng.random(n // 2), rng.integers(-60, 3, size=n // 2))
+    edge = [np.ldexp(m, e) for e in (-1021, -1020, -400, -1, 0, 1, 400, 1019, 1020)
+            for m in (1.0, 1.0 + 2.0**-52, 2.0 - 2.0**-52, 1.5, 1.0 + 2.0**-20, 1.0 + 2.0**-21, 2.0 - 2.0**-21)]
+    x[-len(edge):] = edge
+    xd = torch.as_tensor(x, device=cuda_dev)
+    got, want = torch.empty_like(xd), torch.empty_like(xd)
+    lib = ctypes.CDLL(str(so))
+    p = ctypes.c_void_p
+    assert lib.recip_all(n, p(xd.data_ptr()), p(got.data_ptr()), p(want.data_ptr())) == 0
+    got, want = got.cpu().numpy(), want.cpu().numpy()
+    assert np.all(np.abs(got - want) <= np.spacing(np.abs(want)))
