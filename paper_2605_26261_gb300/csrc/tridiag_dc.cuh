@@ -123,11 +123,19 @@ __host__ __device__ __forceinline__ Span span_of(int i, int s, int m)
     return p;
 }
 
+// Couplings below this are taken as zero (the largest coefficient is about one): they move
+// no eigenvalue by more.  In a block of this scale s the distances between poles and roots
+// are at least s 2^-110, so every reciprocal, and the square of one, stays in range.
+constexpr double kNoCoupling = 0x1p-400;
+
 // Phase 0: leaves of the tearing (w.d and w.e hold the matrix on entry, e[k] couples
 // k and k + 1 and is replaced by its absolute value).
 __host__ __device__ inline void leaf_abs(const Work &w, int t, int T)
 {
-    for (int i = t; i < w.m; i += T) w.e[i] = i + 1 < w.m ? fabs(w.e[i]) : 0.0;
+    for (int i = t; i < w.m; i += T) {
+        const double e = i + 1 < w.m ? fabs(w.e[i]) : 0.0;
+        w.e[i] = e >= kNoCoupling ? e : 0.0;
+    }
 }
 __host__ __device__ inline void leaf_tear(const Work &w, int t, int T)
 {
@@ -439,6 +447,7 @@ __host__ __device__ inline bool secular_root(const Work &w, int lo, int hi, int 
     for (int it = 0; it < kMaxIter; ++it) {
         const Halves<double> h = secular(w, lo, a, hi, c, o, x);
         const double v = irho + h.psi + h.phi;
+        if (v != v) return false;
         if (v < 0.0) lb = x;
         else ub = x;
         tau = x;

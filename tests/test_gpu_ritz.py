@@ -100,6 +100,28 @@ def test_a_chain_does_not_depend_on_the_others(cuda_dev):
         assert np.array_equal(t1[0], th[c]) and np.array_equal(w1[0], w[c])
 
 
+@pytest.mark.parametrize("m", [4, 8, 33, 130])
+@pytest.mark.parametrize("scale", [1e-60, 1e-119, 1e-122, 1e-150, 1e-200, 1e-300, 1e-309])
+def test_blocks_of_scales_far_apart(cuda_dev, m, scale):
+    # a block of coefficients near one and a block of much smaller ones, in either order and
+    # in turn; the tolerances of the file's head
+    rng = np.random.default_rng(m)
+    a, b = rng.normal(size=m), np.abs(rng.normal(size=m)) + 0.1
+    f = np.ones(m)
+    f[m // 2:] = scale
+    turn = np.where(np.arange(m) % 4 < 2, 1.0, scale)
+    probs = [(a * f, b * f), (a * f[::-1], b * f[::-1]), (a * turn, b * turn), (0 * a, b * f), (f, b * f)]
+    th, w = ritz(np.array([p[0] for p in probs]), np.array([p[1] for p in probs]), [m] * len(probs), cuda_dev)
+    for c, (x, y) in enumerate(probs):
+        ev, S = np.linalg.eigh(np.diag(x) + np.diag(y[:m - 1], 1) + np.diag(y[:m - 1], -1))
+        norm = np.abs(ev).max()
+        assert np.abs(th[c] - ev).max() <= 1e-13 * norm, c
+        for beta in (0.0, 1.0, 4.0):
+            g = lambda e: np.exp(-beta * (e - ev[0]) / norm)
+            assert abs((w[c] * g(th[c])).sum() - (S[0] ** 2 * g(ev)).sum()) <= 1e-12, (c, beta)
+    ftlm.ftlm_ritz_status()
+
+
 RECIP = r"""
 #include <cstring>
 #include "tridiag_dc.cuh"
