@@ -377,8 +377,8 @@ ftlm_status ftlm::basis_create_half(int N, int two_sz, int n_bonds, const int *b
     double jsum4 = 0.0;
     for (int k = 0; k < n_bonds; ++k) jsum4 += J[k] / 4.0;
     auto round_up = [](int v) { return (v + kBondChunk - 1) / kBondChunk * kBondChunk; };
-    // host images of the slot arrays: CR and CLT (FP32), rows of doubles, walk A (FP32 and
-    // FP64), walk B
+    // host images of the slot arrays: CR (FP32), rows of doubles, CLT (FP32), whole numbers of
+    // the rows of doubles, walk A (FP32 and FP64), walk B
     std::vector<uint4> slots(7 * (size_t)kMaxBondSlots, make_uint4(0u, 0u, 0u, 0u));
     auto put = [&](int which, int pos, uint32_t mlo, uint32_t mhi, double jh) {
         float f = (float)jh;
@@ -476,6 +476,11 @@ ftlm_status ftlm::basis_create_half(int N, int two_sz, int n_bonds, const int *b
         std::stable_sort(order.begin(), order.end(), [&](int p, int q) {
             return std::min(bi[p], bj[p]) > std::min(bi[q], bj[q]);
         });
+        // Sums of J/2 stay below 2^61 units of at least 2^-1074 (the sum of |J| itself may be out
+        // of range, and the unit's inverse)
+        double js = 0.0;
+        for (int k = 0; k < n_bonds; ++k) js += std::fabs(J[k]) * 0x1p-10;
+        const int shift = js > 0.0 ? std::min(1074, 50 - std::ilogb(js)) : 1074;
         for (int pos = 0; pos < n_bonds; ++pos) {
             const int k = order[pos];
             const uint64_t m = (1ull << bi[k]) | (1ull << bj[k]);
@@ -484,13 +489,11 @@ ftlm_status ftlm::basis_create_half(int N, int two_sz, int n_bonds, const int *b
             std::memcpy(&db, &jh, 8);
             slots[(size_t)kMaxBondSlots + pos] =
                 make_uint4((uint32_t)m, (uint32_t)(m >> 32), (uint32_t)db, (uint32_t)(db >> 32));
+            const long long f = std::llrint(std::ldexp(jh, shift));
+            std::memcpy(reinterpret_cast<char *>(&slots[3 * (size_t)kMaxBondSlots]) + 8 * pos, &f, 8);
         }
-        // sums of J/2 stay below 2^61 units
-        const int e = jabs > 0.0 ? std::ilogb(jabs) + 1 : 0;
-        const int shift = std::min(1000, 61 - e);
         for (BondList *c : {&b->bonds_cr, &b->bonds_clt}) {
             c->n64 = n_bonds;
-            c->jscale = std::ldexp(1.0, shift);
             c->junscale = std::ldexp(1.0, -shift);
         }
     }
@@ -614,6 +617,7 @@ ftlm_status ftlm::basis_create_half(int N, int two_sz, int n_bonds, const int *b
     b->bonds_cr.slots_f64 = b->bond_slots + kMaxBondSlots;
     b->bonds_clt.slots_f32 = b->bond_slots + 2 * kMaxBondSlots;
     b->bonds_clt.slots_f64 = b->bonds_cr.slots_f64;
+    b->bonds_cr.whole_f64 = b->bonds_clt.whole_f64 = reinterpret_cast<const long long *>(b->bond_slots + 3 * kMaxBondSlots);
 
     // The copy returns once the image is staged, so `image` may go out of scope;
     // the kernels below follow it in stream order.

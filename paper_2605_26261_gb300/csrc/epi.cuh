@@ -75,8 +75,9 @@ inline EpiDev epi_of(const LanczosHv *epi)
         ep.fixed = epi->fixed;
         // |alpha_j| <= ||H|| < 2^e, and ||y|| <= 2 ||H||: the tiles' sums together stay
         // below 2^50 units in magnitude, whatever their number (two_word.cuh for their rests)
-        const int e = epi->norm_bound > 0.0 ? std::ilogb(epi->norm_bound) + 1 : 0;
-        const int shift = std::min(1000, 49 - e);
+        // (a bound out of range, at either end, does not put alpha there)
+        const double nb = epi->norm_bound;
+        const int shift = !std::isfinite(nb) ? 49 - 1025 : nb > 0.0 ? std::min(1000, 48 - std::ilogb(nb)) : 1000;
         ep.scale = std::ldexp(1.0, shift);
         ep.unscale = std::ldexp(1.0, -shift);
         ep.alpha_stride = epi->alpha_stride;

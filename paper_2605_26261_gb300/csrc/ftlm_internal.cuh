@@ -47,9 +47,10 @@ struct BondList {
     // FP64 rows (row_f64): n64 bonds with their full masks, in the order of their lower
     // site, highest first
     const uint4 *slots_f64;  // J/2 as double in .z (low word), .w (high word)
+    const long long *whole_f64;  // J/2 of the same bonds as a whole number of units
     int n64;
     int pad64;
-    double jscale, junscale;  // 2^jshift and its inverse: J/2 as a whole number
+    double junscale;  // the unit
 };
 
 // Scalars of one Lanczos chain, kept on the device between launches.  The stored
@@ -184,7 +185,7 @@ struct ftlm_basis {
     int n_hi_bonds;                // high-high bonds (walk B of the split H.v)
     double jsum4_hi;               // their sum of J_b / 4
     void *block;        // one pooled device allocation holding every table below
-    uint4 *bond_slots;  // device: cr f32, rows of doubles, clt f32, unused, walk-A f32, walk-A f64
+    uint4 *bond_slots;  // device: cr f32, rows of doubles, clt f32, whole_f64, walk-A f32, walk-A f64
                         // (LoWalk layout), walk-B bonds (kMaxBondSlots each)
     uint32_t *uhi;      // CR: high patterns grouped by popcount, ascending (walk B)
     uint32_t *lo_tiles; // CR: walk A tile table of the split H.v (LoWalk), or null

@@ -188,7 +188,7 @@ __device__ __forceinline__ void rows_clt(const SectorTables &s, const BondList &
 // bonds of its own: a bit mask per lane (integer work), from which every lane takes its
 // next bond, so that a pass over B chains costs as many FMAs as the warp's longest
 // list has entries (about 60 % of the bonds) instead of one per bond.  The diagonal is
-// summed as a whole number (J/2 in units of 2^-jshift, exact to 2^-62 sum |J|) instead
+// summed as a whole number (J/2 in units of junscale, exact to 2^-62 sum |J|) instead
 // of one FP64 addition per bond and row.  The bonds come in the order of their lower
 // site, highest first: those above the bits that differ inside a warp are antiparallel
 // in all lanes or in none, so the lanes take them together and gather contiguous rows.
@@ -198,7 +198,7 @@ __device__ __forceinline__ void rows_clt(const SectorTables &s, const BondList &
 template <typename Lbl> struct BondLists {
     Lbl m[kMaxBondSlots];        // both site bits
     double j[kMaxBondSlots];     // J / 2
-    long long f[kMaxBondSlots];  // J / 2 in units of 2^-jshift
+    long long f[kMaxBondSlots];  // J / 2 in units of bl.junscale
 };
 
 template <typename Lbl>
@@ -210,7 +210,7 @@ __device__ __forceinline__ void stage_lists(const BondList &bl, BondLists<Lbl> &
         if constexpr (sizeof(Lbl) == 8) m |= (Lbl)e.y << 32;
         s.m[i] = m;
         s.j[i] = slot_jh<double>(e);
-        s.f[i] = (long long)rint(s.j[i] * bl.jscale);
+        s.f[i] = bl.whole_f64[i];
     }
 }
 

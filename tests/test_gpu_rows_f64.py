@@ -96,3 +96,36 @@ def test_couplings_far_from_one(cuda_dev, scale):
             with ftlm.Basis(N, 0, (bi, bj, J * root), mode) as d:
                 a = ftlm.lanczos(d, 4, 8, seed=2, dtype=torch.float64, keep_coeffs=True)["alpha"] / root
                 assert torch.abs(a - ref).max().item() <= 1e-10 * torch.abs(ref).max().item()
+
+
+@pytest.mark.parametrize("mode", [ftlm.RANK_CLT, ftlm.RANK_CR])
+def test_couplings_whose_sum_of_magnitudes_overflows(cuda_dev, mode):
+    # sum |J| = 3.2e308 is out of range, H and its rows are not
+    N, scale = 8, 4e307
+    bi, bj, J = inputs.ring(N)
+    J = J * np.linspace(0.5, 1.0, N)
+    with ftlm.Basis(N, 0, (bi, bj, J), mode) as b, ftlm.Basis(N, 0, (bi, bj, J * scale * 4 / 3), mode) as c:
+        x = torch.randn(b.dim, device=cuda_dev, dtype=torch.float64) / 16
+        y, z = torch.empty_like(x), torch.empty_like(x)
+        ftlm.ftlm_hv(b.handle, x, y)
+        ftlm.ftlm_hv(c.handle, x, z)
+        assert torch.isfinite(z).all()
+        assert torch.abs(z / (scale * 4 / 3) - y).max().item() <= 1e-13 * torch.abs(y).max().item()
+        ref = ftlm.lanczos(b, 4, 3, seed=2, dtype=torch.float64, keep_coeffs=True)
+        got = ftlm.lanczos(c, 4, 3, seed=2, dtype=torch.float64, keep_coeffs=True)
+        a, g = ref["alpha"][:, 0], got["alpha"][:, 0] / (scale * 4 / 3)
+        assert torch.abs(g - a).max().item() <= 1e-12 * torch.abs(ref["alpha"]).max().item()
+
+
+@pytest.mark.parametrize("mode", [ftlm.RANK_CLT, ftlm.RANK_CR])
+@pytest.mark.parametrize("scale", [2.0 ** -930, 2.0 ** -960, 2.0 ** -990, 2.0 ** 1000])
+def test_couplings_near_the_ends_of_the_range(cuda_dev, mode, scale):
+    # the unit of the whole-number diagonal has no inverse in range below about 2^-960
+    N = 12
+    bi, bj, J = inputs.random_graph(N, seed=8)
+    with ftlm.Basis(N, 0, (bi, bj, J), mode) as b, ftlm.Basis(N, 0, (bi, bj, J * scale), mode) as c:
+        x = torch.randn(b.dim, device=cuda_dev, dtype=torch.float64)
+        y, z = torch.empty_like(x), torch.empty_like(x)
+        ftlm.ftlm_hv(b.handle, x, y)
+        ftlm.ftlm_hv(c.handle, x, z)
+        assert torch.abs(z / scale - y).max().item() <= 1e-13 * torch.abs(y).max().item()
