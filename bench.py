@@ -1098,8 +1098,8 @@ def serve_stream(n_jobs, steps_per_poll, warmup, local=0, clocks=None, live_rows
     alone_s = time.perf_counter() - t0
 
     # the same jobs through the plain per-sector path of the library, one job at a
-    # time: ftlm.run_ftlm (each sector through ftlm_lanczos in turn, then the sums),
-    # results read back per job
+    # time: ftlm.run_ftlm (each sector through ftlm_lanczos, small ones side by side over
+    # four streams, then the sums), results read back per job
     plain_jobs, _ = serve.poisson_jobs(n_jobs, 200.0, seed=4)
     Td = torch.as_tensor(T, device=torch.device("cuda", local))
     t0 = time.perf_counter()
@@ -1180,8 +1180,8 @@ def run_serving(args):
                           "p99_ms": sv["one_at_a_time_p99_ms"],
                           "note": "same jobs and engine, one job in flight at a time, all queued at t=0"},
         "plain_one_at_a_time": {"jobs_per_s": sv["plain_one_at_a_time_jobs_per_s"],
-                                "note": "same jobs through ftlm.run_ftlm (every sector through ftlm_lanczos in turn, "
-                                        "then the sums), one job at a time"},
+                                "note": "same jobs through ftlm.run_ftlm (every sector through ftlm_lanczos, small ones "
+                                        "side by side over four streams, then the sums), one job at a time"},
         "identical_alone_vs_mix": sv["identical_alone_vs_mix"],
         "max_rel_diff_alone_vs_mix": sv["max_rel_diff_alone_vs_mix"],
         "engine": {k: sv[k] for k in ("max_jobs_in_flight", "max_units", "polls", "host_s")},

@@ -218,7 +218,7 @@ __device__ __forceinline__ RitzIo ritz_io(int c, int M, const int *mv, double *t
 // non-finite coefficient or an unconverged root gets NaN Ritz values and weights.
 //
 // Bound: FP64 instructions on one SM per chain (two lanes per cycle).  One thread per
-// root of the merge; the whole problem lives in shared memory (88 bytes per row).
+// root of the merge; the whole problem lives in shared memory (dc::kBytesPerRow, 108).
 __global__ void __launch_bounds__(kRitzThreads)
 ritz_dc_kernel(int M, const double *__restrict__ alpha, const double *__restrict__ beta, const int *__restrict__ mv,
                double *theta, double *weight, const RitzRow *rows)

@@ -18,28 +18,6 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;  // use lane 0's value: lanes may differ in the last bit
 }
 
-// Sum over the block; the result is valid in thread 0.
-template <int THREADS>
-__device__ __forceinline__ double block_sum(double v)
-{
-    __shared__ double sh[THREADS / 32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    v = warp_sum(v);
-    if (lane == 0) sh[w] = v;
-    __syncthreads();
-    double r = 0.0;
-    if (w == 0) {
-        r = (lane < THREADS / 32) ? sh[lane] : 0.0;
-        r = warp_sum(r);
-    }
-    __syncthreads();
-    return r;
-}
-
-}  // namespace ftlm
-
-namespace ftlm {
-
 // Per-thread accumulator of dot-product terms a * b.  For FP32 operands every
 // product is split exactly into p + e (p = fl(a b), e = fma(a, b, -p)) and added
 // to a two-float sum (hi, lo) with the error-free TwoSum of Knuth, so the running

@@ -447,10 +447,10 @@ __host__ __device__ inline bool secular_root(const Work &w, int lo, int hi, int 
     for (int it = 0; it < kMaxIter; ++it) {
         const Halves<double> h = secular(w, lo, a, hi, c, o, x);
         const double v = irho + h.psi + h.phi;
+        tau = x;
         if (v != v) return false;
         if (v < 0.0) lb = x;
         else ub = x;
-        tau = x;
         // rounding level of f at x (Gu & Eisenstat's stopping rule)
         const bool small = fabs(v) <= 0x1p-52 * n * (irho + fabs(h.psi) + fabs(h.phi));
         const double da = (w.d[a] - dorg) - x, db = (w.d[b] - dorg) - x;
