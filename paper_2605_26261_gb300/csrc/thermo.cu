@@ -105,9 +105,10 @@ thermo_kernel(const ThermoArgs a, const double *__restrict__ T, double *E, doubl
         s_a2[FTLM_MAX_SECTORS], s_G[FTLM_MAX_SECTORS][2];
     cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
     const unsigned lane = threadIdx.x & 31u;
-    const int per_sector = a.R * a.M;
-    const int first = (int)cl.block_rank() * kThermoThreads + (int)threadIdx.x;  // pairs first, first + 256 C, ...
-    constexpr int kStep = kThermoThreads * C;
+    // unsigned: with up to 2^31 - 1 pairs the index of a thread's last step passes 2^31
+    const unsigned M = (unsigned)a.M, per_sector = (unsigned)a.R * M;
+    const unsigned first = cl.block_rank() * kThermoThreads + threadIdx.x;  // pairs first, first + 256 C, ...
+    constexpr unsigned kStep = kThermoThreads * C;
     const double beta = 1.0 / T[blockIdx.x / C];
     const long long inf_key = dc::order_key(INFINITY);
 
@@ -119,9 +120,9 @@ thermo_kernel(const ThermoArgs a, const double *__restrict__ T, double *E, doubl
     for (int s = 0; s < a.ns; ++s) {
         long long m = inf_key;
         int any = 0;
-        for (int i = first; i < per_sector; i += kStep) {
-            const int r = i / a.M;
-            if (i - r * a.M >= __ldg(a.meff[s] + r)) continue;
+        for (unsigned i = first; i < per_sector; i += kStep) {
+            const unsigned r = i / M;
+            if ((int)(i - r * M) >= __ldg(a.meff[s] + r)) continue;
             m = min(m, dc::order_key(__ldg(a.theta[s] + i)));
             any = 1;
         }
@@ -152,10 +153,10 @@ thermo_kernel(const ThermoArgs a, const double *__restrict__ T, double *E, doubl
     for (int s = 0; s < a.ns; ++s) {
         const double t = s_t[s];
         double x0 = 0.0, x1 = 0.0;
-        for (int i = first; i < per_sector; i += kStep) {
-            const int r = i / a.M;
+        for (unsigned i = first; i < per_sector; i += kStep) {
+            const unsigned r = i / M;
             double p = 0.0;
-            if (i - r * a.M < __ldg(a.meff[s] + r)) {
+            if ((int)(i - r * M) < __ldg(a.meff[s] + r)) {
                 const double x = __ldg(a.theta[s] + i) - t;
                 p = __ldg(a.weight[s] + i) * exp(-beta * x);
                 x0 += p;
@@ -181,9 +182,9 @@ thermo_kernel(const ThermoArgs a, const double *__restrict__ T, double *E, doubl
     for (int s = 0; s < a.ns; ++s) {
         const double t = s_t[s], mu = s_mu[s];
         double x2 = 0.0;
-        for (int i = first; i < per_sector; i += kStep) {
-            const int r = i / a.M;
-            if (i - r * a.M < __ldg(a.meff[s] + r)) {
+        for (unsigned i = first; i < per_sector; i += kStep) {
+            const unsigned r = i / M;
+            if ((int)(i - r * M) < __ldg(a.meff[s] + r)) {
                 const double x = __ldg(a.theta[s] + i) - t;
                 const double p = STORE ? s_p[slot] : __ldg(a.weight[s] + i) * exp(-beta * x);
                 const double d = x - mu;

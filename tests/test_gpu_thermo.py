@@ -95,3 +95,22 @@ def test_an_unconverged_chain_shows_in_every_observable(cuda_dev, whole_sector):
     got = ftlm.thermo(dev, torch.tensor([0.1, 1.0], device=cuda_dev, dtype=torch.float64), 6, 20)
     for k in ("E", "C", "chi"):
         assert torch.isnan(got[k]).all()
+
+
+def test_as_many_pairs_as_are_accepted(cuda_dev):
+    # 2^31 - 2 pairs: the index of a thread's last step passes 2^31.  Two chains have pairs, the
+    # first and the last.
+    M, R = 1023, 2099202
+    rng = np.random.default_rng(1)
+    th, w = (torch.zeros((R, M), dtype=torch.float64, device=cuda_dev) for _ in range(2))
+    m = torch.zeros(R, dtype=torch.int32, device=cuda_dev)
+    secs = []
+    for r in (0, R - 1):
+        t, x = np.sort(rng.uniform(-6.0, 4.0, size=(1, M))), rng.random((1, M))
+        th[r], w[r], m[r] = torch.as_tensor(t[0]), torch.as_tensor(x[0]), M
+        secs.append((0, R, t, x, np.array([M])))
+    T = np.array([0.3, 2.0])
+    got = ftlm.thermo([(0, R, {"theta": th, "weight": w, "m_eff": m})], torch.as_tensor(T, device=cuda_dev), R, M)
+    ref = reference(secs, T, 1, 2.0, 0.0, True)
+    for k in ("E", "C"):
+        assert np.abs(got[k].cpu().numpy() - ref[k]).max() <= 1e-12 * np.abs(ref[k]).max(), k
